@@ -1,21 +1,128 @@
-// Kendall discordant-pair counts for the MMD test of Sec. 5 (Mallows kernel).
+// The GPU side of the MMD test of Sec. 5 (Mallows kernel): Kendall
+// discordant-pair counts of pairs of permutations, and the inversion of slot
+// orders.
 //
 // For each pair p of permutations (s, t) = (perms[2p], perms[2p + 1]) of
-// [0, n), n_dis = #{i < j : (s_i < s_j) != (t_i < t_j)}.  One CTA owns one
-// pair at a time: both permutations are staged in shared memory, every
-// thread takes rows i (strided) and counts the discordant j > i, and a block
-// reduction gives the count.  O(n^2) comparisons per pair, all in shared
-// memory; the pairs are independent.
+// [0, n), n_dis = #{i < j : (s_i < s_j) != (t_i < t_j)}.  Ordered by s, the
+// pair becomes one sequence c (c[s_i] = t_i) and n_dis its inversions.  One
+// warp owns one pair at a time and walks c 32 elements a step: the inversions
+// with earlier steps are the set bits above the element in a shared-memory
+// bitmap of the values seen (a count of the words above it and a population
+// count of its own word), those inside the step come from one ballot per
+// value bit.  About 75 warp instructions per 32 elements, so n^2 / 32 bit
+// operations in all where comparing every pair in shared memory took n^2 / 2
+// comparisons and was bound by the shared-memory loads (96 % busy): 50,000
+// pairs of length 1000 on GB300: 5.53 -> 0.47 ms.
+// Rows that are not permutations of [0, n) have no such sequence: their pairs
+// are marked and counted by the all-pairs kernel, one CTA each.
+#include <atomic>
 #include <cstdint>
+
+#include "bshuffle_device.cuh"
 
 #include "bshuffle_internal.h"
 
 namespace bsh {
 namespace {
 
-constexpr int kKBlock = 256;
-constexpr uint32_t kMaxN = 4096;
+using dev::kFull;
 
+constexpr int kKBlock = 256;
+constexpr int kKWarps = kKBlock / 32;
+constexpr uint32_t kMaxN = 4096;
+constexpr uint64_t kNotPermutations = ~uint64_t{0};  // above every count (n_dis < 2^23)
+
+// Shared memory of one warp of the inversion count: the sequence c (16-bit),
+// the bitmap of the values seen and the set bits above each of its words.
+__host__ __device__ constexpr uint32_t kendall_words(uint32_t n) { return (n + 1023u) / 1024u * 32u; }
+__host__ __device__ constexpr uint32_t kendall_warp_bytes(uint32_t n)
+{
+    return (n + 31u) / 32u * 64u + 2u * kendall_words(n) * 4u;
+}
+
+__global__ void __launch_bounds__(kKBlock) kendall_inversions_kernel(const uint32_t *__restrict__ perms, uint32_t n,
+                                                                     uint32_t value_bits, uint64_t pairs,
+                                                                     uint64_t *__restrict__ out)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint32_t lt = dev::lanemask_lt();
+    const uint32_t words = kendall_words(n);
+    unsigned char *mine = s_raw + warp * kendall_warp_bytes(n);
+    uint32_t *bits = reinterpret_cast<uint32_t *>(mine);
+    uint32_t *above = bits + words;
+    uint16_t *c = reinterpret_cast<uint16_t *>(above + words);
+
+    for (uint64_t p = uint64_t{blockIdx.x} * kKWarps + warp; p < pairs; p += uint64_t{gridDim.x} * kKWarps) {
+        const uint32_t *a = perms + 2 * p * n;
+        const uint32_t *b = a + n;
+        for (uint32_t w = lane; w < words; w += 32) bits[w] = 0u;
+        __syncwarp();
+        bool ok = true;
+#pragma unroll 4
+        for (uint32_t i = lane; i < n; i += 32) {
+            const uint32_t s = a[i], t = b[i];
+            if (s < n && t < n) {
+                const uint32_t old = atomicOr(&bits[s >> 5], 1u << (s & 31u));
+                ok = ok && ((old >> (s & 31u)) & 1u) == 0u;
+                c[s] = static_cast<uint16_t>(t);
+            } else {
+                ok = false;
+            }
+        }
+        if (!__all_sync(kFull, ok)) {
+            if (lane == 0) out[p] = kNotPermutations;
+            __syncwarp();
+            continue;
+        }
+        __syncwarp();
+        for (uint32_t w = lane; w < words; w += 32) {
+            bits[w] = 0u;
+            above[w] = 0u;
+        }
+        __syncwarp();
+        uint32_t count = 0;
+        for (uint32_t first = 0; first < n; first += 32) {
+            const bool live = first + lane < n;  // lanes past the end come after every live one
+            const uint32_t v = live ? c[first + lane] : 0u;
+            const uint32_t w = v >> 5;
+            if (live) count += above[w] + static_cast<uint32_t>(__popc(bits[w] & (0xfffffffeu << (v & 31u))));
+            // lanes whose value is greater: the first differing bit decides
+            uint32_t greater = 0, equal = kFull;
+            for (uint32_t bit = value_bits; bit-- > 0u;) {
+                const bool one = (v >> bit) & 1u;
+                const uint32_t ones = __ballot_sync(kFull, one);
+                if (!one) greater |= equal & ones;
+                equal &= one ? ones : ~ones;
+            }
+            if (live) count += static_cast<uint32_t>(__popc(greater & lt));
+            __syncwarp();
+            if (live) {
+                const uint32_t old = atomicOr(&bits[w], 1u << (v & 31u));
+                ok = ok && ((old >> (v & 31u)) & 1u) == 0u;
+            }
+            __syncwarp();
+            uint32_t higher = 0;  // set bits of the words after these 32
+            for (uint32_t q = words; q > 0u; q -= 32u) {
+                const uint32_t pc = static_cast<uint32_t>(__popc(bits[q - 32u + lane]));
+                uint32_t sum = pc;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t u = __shfl_down_sync(kFull, sum, d);
+                    if (lane + static_cast<uint32_t>(d) < 32u) sum += u;
+                }
+                above[q - 32u + lane] = higher + sum - pc;
+                higher += __shfl_sync(kFull, sum, 0);
+            }
+            __syncwarp();
+        }
+        count = __reduce_add_sync(kFull, count);
+        ok = __all_sync(kFull, ok);
+        if (lane == 0) out[p] = ok ? count : kNotPermutations;
+    }
+}
+
+// Every pair i < j compared, for the pairs of rows marked as no permutations.
 __global__ void __launch_bounds__(kKBlock) kendall_pairs_kernel(const uint32_t *__restrict__ perms, uint32_t n,
                                                                 uint64_t pairs, uint64_t *__restrict__ out)
 {
@@ -23,36 +130,42 @@ __global__ void __launch_bounds__(kKBlock) kendall_pairs_kernel(const uint32_t *
     __shared__ uint32_t s_b[kMaxN];
     __shared__ unsigned long long s_sum[kKBlock / 32];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    for (uint64_t p = blockIdx.x; p < pairs; p += gridDim.x) {
-        const uint32_t *a = perms + 2 * p * n;
-        const uint32_t *b = a + n;
-        for (uint32_t i = tid; i < n; i += kKBlock) {
-            s_a[i] = a[i];
-            s_b[i] = b[i];
-        }
-        __syncthreads();
-        unsigned long long count = 0;
-        // rows i and n-1-i together keep the work per thread balanced
-        for (uint32_t i = tid; i < (n + 1) / 2; i += kKBlock) {
-            for (uint32_t r = 0; r < 2; ++r) {
-                const uint32_t row = r == 0 ? i : n - 1 - i;
-                if (r == 1 && row == i) break;
-                const uint32_t ai = s_a[row], bi = s_b[row];
-                uint32_t c = 0;
-                for (uint32_t j = row + 1; j < n; ++j) c += ((ai < s_a[j]) != (bi < s_b[j])) ? 1u : 0u;
-                count += c;
+    for (uint64_t p0 = uint64_t{blockIdx.x} * kKBlock; p0 < pairs; p0 += uint64_t{gridDim.x} * kKBlock) {
+        const bool marked = p0 + tid < pairs && out[p0 + tid] == kNotPermutations;
+        if (!__syncthreads_or(marked)) continue;
+        const uint64_t p1 = p0 + kKBlock < pairs ? p0 + kKBlock : pairs;
+        for (uint64_t p = p0; p < p1; ++p) {
+            if (!__syncthreads_or(marked && p == p0 + tid)) continue;
+            const uint32_t *a = perms + 2 * p * n;
+            const uint32_t *b = a + n;
+            for (uint32_t i = tid; i < n; i += kKBlock) {
+                s_a[i] = a[i];
+                s_b[i] = b[i];
             }
-        }
+            __syncthreads();
+            unsigned long long count = 0;
+            // rows i and n-1-i together keep the work per thread balanced
+            for (uint32_t i = tid; i < (n + 1) / 2; i += kKBlock) {
+                for (uint32_t r = 0; r < 2; ++r) {
+                    const uint32_t row = r == 0 ? i : n - 1 - i;
+                    if (r == 1 && row == i) break;
+                    const uint32_t ai = s_a[row], bi = s_b[row];
+                    uint32_t c = 0;
+                    for (uint32_t j = row + 1; j < n; ++j) c += ((ai < s_a[j]) != (bi < s_b[j])) ? 1u : 0u;
+                    count += c;
+                }
+            }
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) count += __shfl_down_sync(0xffffffffu, count, d);
-        if (lane == 0) s_sum[warp] = count;
-        __syncthreads();
-        if (tid == 0) {
-            unsigned long long total = 0;
-            for (int w = 0; w < kKBlock / 32; ++w) total += s_sum[w];
-            out[p] = total;
+            for (int d = 16; d > 0; d >>= 1) count += __shfl_down_sync(kFull, count, d);
+            if (lane == 0) s_sum[warp] = count;
+            __syncthreads();
+            if (tid == 0) {
+                unsigned long long total = 0;
+                for (int w = 0; w < kKBlock / 32; ++w) total += s_sum[w];
+                out[p] = total;
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
 
@@ -95,8 +208,25 @@ cudaError_t launch_kendall_pairs(const uint32_t *perms, uint32_t n, uint64_t pai
     cudaError_t e = cudaGetDevice(&device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
-    const uint64_t grid = pairs < static_cast<uint64_t>(sms) * 8 ? pairs : static_cast<uint64_t>(sms) * 8;
-    kendall_pairs_kernel<<<static_cast<unsigned>(grid), kKBlock, 0, stream>>>(perms, n, pairs, out);
+    if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+    static std::atomic<bool> configured[64];  // attribute set on this device
+    if (!configured[device].load(std::memory_order_acquire)) {
+        e = cudaFuncSetAttribute(kendall_inversions_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(kKWarps * kendall_warp_bytes(kMaxN)));
+        if (e != cudaSuccess) return e;
+        configured[device].store(true, std::memory_order_release);
+    }
+    uint32_t value_bits = 0;
+    while ((1u << value_bits) < n) ++value_bits;
+    const uint64_t most = static_cast<uint64_t>(sms) * 8;
+    const uint64_t blocks = (pairs + kKWarps - 1) / kKWarps;
+    kendall_inversions_kernel<<<static_cast<unsigned>(blocks < most ? blocks : most), kKBlock,
+                                kKWarps * kendall_warp_bytes(n), stream>>>(perms, n, value_bits, pairs, out);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const uint64_t checks = (pairs + kKBlock - 1) / kKBlock;
+    kendall_pairs_kernel<<<static_cast<unsigned>(checks < most ? checks : most), kKBlock, 0, stream>>>(perms, n, pairs,
+                                                                                                      out);
     return cudaGetLastError();
 }
 
