@@ -289,11 +289,14 @@ int bshuffle_window_scatter(const void *in, void *out, uint64_t n, uint32_t elem
  * kernel exp(-lambda n_dis / C(n, 2)); 1 <= n <= 4096.
  * bshuffle_invert_rows: sigma[r][idx[r][j]] = j for each of `rows` rows of
  * length n: the slot order of a shuffle (slot j holds element idx[j]) turned
- * into each element's rank, the convention of Sec. 2.  Device pointers;
- * asynchronous on `stream`.
+ * into each element's rank, the convention of Sec. 2.
+ * bshuffle_sample_ranks: row r of sigma (rows x n) = those ranks for the
+ * shuffle of length n with seed seed0 + r (mod 2^64), without the slot order
+ * in between; 1 <= n <= 4096.  Device pointers; asynchronous on `stream`.
  */
 int bshuffle_kendall_pairs(const uint32_t *perms, uint32_t n, uint64_t num_pairs, uint64_t *out, void *stream);
 int bshuffle_invert_rows(const uint32_t *idx, uint32_t n, uint64_t rows, uint32_t *sigma, void *stream);
+int bshuffle_sample_ranks(uint64_t n, uint64_t rows, uint64_t seed0, uint32_t rounds, uint32_t *sigma, void *stream);
 
 /*
  * Synchronises `stream`, then returns and clears the first device-side error

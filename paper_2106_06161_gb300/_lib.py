@@ -80,6 +80,7 @@ SIGNATURES = {
     "bshuffle_permute_ablation": (_int, [_p, _p, _u64, _u32, _u64, _u32, _int, _p]),
     "bshuffle_kendall_pairs": (_int, [_p, _u32, _u64, _p, _p]),
     "bshuffle_invert_rows": (_int, [_p, _u32, _u64, _p, _p]),
+    "bshuffle_sample_ranks": (_int, [_u64, _u64, _u64, _u32, _p, _p]),
 }
 
 _lock = threading.Lock()
@@ -305,6 +306,11 @@ def bshuffle_kendall_pairs(perms_ptr: int, n: int, num_pairs: int, out_ptr: int,
 
 def bshuffle_invert_rows(idx_ptr: int, n: int, rows: int, sigma_ptr: int, stream: int = 0) -> None:
     _check(load().bshuffle_invert_rows(idx_ptr, n, rows, sigma_ptr, stream), "bshuffle_invert_rows")
+
+
+def bshuffle_sample_ranks(n: int, rows: int, seed0: int, rounds: int, sigma_ptr: int, stream: int = 0) -> None:
+    _check(load().bshuffle_sample_ranks(n, rows, seed0 & (2**64 - 1), rounds, sigma_ptr, stream),
+           "bshuffle_sample_ranks")
 
 
 def bshuffle_version() -> int:

@@ -821,6 +821,18 @@ int bshuffle_invert_rows(const uint32_t *idx, uint32_t n, uint64_t rows, uint32_
     return e == cudaSuccess ? BSHUFFLE_OK : cuda_fail(e);
 }
 
+int bshuffle_sample_ranks(uint64_t n, uint64_t rows, uint64_t seed0, uint32_t rounds, uint32_t *sigma, void *stream)
+{
+    if (rounds > BSHUFFLE_MAX_ROUNDS) return BSHUFFLE_ERR_ROUNDS;
+    if (rows == 0) return BSHUFFLE_OK;
+    if (sigma == nullptr) return BSHUFFLE_ERR_NULL;
+    if (n == 0 || n > bsh::kendall_max_n()) return BSHUFFLE_ERR_INVALID;
+    if (reinterpret_cast<uintptr_t>(sigma) % 4 != 0) return BSHUFFLE_ERR_ALIGN;
+    const cudaError_t e =
+        bsh::launch_sample_ranks(geometry_of(n), rounds, seed0, rows, sigma, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? BSHUFFLE_OK : cuda_fail(e);
+}
+
 int bshuffle_get_error(void *stream_ptr)
 {
     cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);

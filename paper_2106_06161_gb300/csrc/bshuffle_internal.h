@@ -235,6 +235,9 @@ cudaError_t launch_ablation(const AblationArgs &a, uint32_t elem_bytes, int vari
 // ------------------------------------------------------------------ statistics (Sec. 5)
 
 uint32_t kendall_max_n();
+// Ranks of `rows` shuffles of length g.n <= kendall_max_n(), seeds seed0 + row.
+cudaError_t launch_sample_ranks(const Geometry &g, uint32_t rounds, uint64_t seed0, uint64_t rows, uint32_t *sigma,
+                                cudaStream_t stream);
 cudaError_t launch_kendall_pairs(const uint32_t *perms, uint32_t n, uint64_t pairs, uint64_t *out,
                                  cudaStream_t stream);
 cudaError_t launch_invert_rows(const uint32_t *idx, uint32_t n, uint64_t rows, uint32_t *sigma, cudaStream_t stream);

@@ -17,16 +17,22 @@ from . import _lib
 
 LAMBDA = 5.0   # the Mallows kernel parameter used throughout Sec. 5
 ALPHA = 0.05
+MAX_RANKS_N = 4096  # longest row that bshuffle_sample_ranks writes
 
 
 def sample_ranks(n: int, count: int, seed0: int = 0, rounds: int = 24) -> torch.Tensor:
     """count permutations of [0, n) as ranks sigma (Sec. 2), seeds seed0, seed0+1, ...
 
-    One batched launch shuffles `count` copies of 0..n-1 (slot order), then
-    each row is inverted into ranks.  Returns a (count, n) int32 CUDA tensor.
+    Up to n = 4096 one kernel writes the ranks; longer rows come from one
+    batched launch over `count` copies of 0..n-1 (slot order), each row then
+    inverted into ranks.  Returns a (count, n) int32 CUDA tensor.
     """
     from . import batched_packed
     dev = torch.device("cuda", torch.cuda.current_device())
+    if 0 < n <= MAX_RANKS_N and count > 0:
+        sigma = torch.empty(count, n, dtype=torch.int32, device=dev)
+        _lib.bshuffle_sample_ranks(n, count, seed0, rounds, sigma.data_ptr(), torch.cuda.current_stream().cuda_stream)
+        return sigma
     iota = torch.arange(n, dtype=torch.int32, device=dev).repeat(count)
     idx = batched_packed(iota, np.full(count, n), [seed0 + t for t in range(count)], rounds)
     sigma = torch.empty_like(idx)

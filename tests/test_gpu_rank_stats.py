@@ -65,3 +65,22 @@ def test_marked_pairs_among_many(st):
         rows[2 * p, 3] = rows[2 * p, 4]
     want = [_discordant(rows[2 * p], rows[2 * p + 1]) for p in range(pairs)]
     assert _counts(st, rows).tolist() == want
+
+
+@pytest.mark.parametrize("n", [1, 2, 15, 16, 17, 255, 256, 257, 1025, 4096, 4097])
+def test_sampled_ranks(st, n):
+    # 4,096 is the longest row of the one-kernel form
+    for seed0, rounds in ((3, 24), (2**64 - 2, 24), (3, 5)):
+        got = st.sample_ranks(n, 6, seed0, rounds).cpu().numpy()
+        assert got.dtype == np.int32 and got.shape == (6, n)
+        for r in range(6):
+            idx = oracle.indices(n, (seed0 + r) % 2**64, rounds)
+            assert np.array_equal(got[r][idx], np.arange(n)), (seed0, rounds, r)
+
+
+def test_sampled_ranks_of_nothing(st):
+    assert st.sample_ranks(7, 0).shape == (0, 7)
+    with pytest.raises(Exception):
+        st.sample_ranks(0, 3)
+    with pytest.raises(Exception):
+        st.sample_ranks(10, 3, rounds=65)
