@@ -416,7 +416,8 @@ int bshuffle_tuning_selected(uint32_t elem_bytes);
  * elements) or BSHUFFLE_KERNEL_BATCHED (the persistent kernel of
  * bshuffle_batched for 4-, 8- and 16-byte elements).  Configuration c has
  * `threads` per CTA (the pipelined shapes: compute warps plus one look-back
- * warp), `items` domain indices per compute thread, the resident CTAs per SM
+ * warp), `items` domain indices per compute thread and tile (batched shapes of
+ * 16: 12 for 8- and 16-byte elements), the resident CTAs per SM
  * its register budget targets (0: not set) and the rounds unrolled at compile
  * time (24: the default count runs unrolled, other counts in a loop; 0: every
  * count runs in a loop).  Configuration 0 is the default.  Every

@@ -155,6 +155,7 @@ int acquire_workspace(cudaStream_t stream, uint64_t words, Workspace **out)
     const uint64_t cap_words = round_up_pow2(words < kMinStatusWords ? kMinStatusWords : words);
     WsHeader keep{};
     keep.tag = 1;
+    keep.batch_tag = 1;
     if (ws.base != nullptr) {
         e = cudaStreamSynchronize(stream);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -505,11 +506,13 @@ int bshuffle_batched(const bshuffle_desc *d_descs, uint32_t count, uint32_t elem
     int rc = acquire_workspace(s, kMinStatusWords, &ws);
     if (rc != BSHUFFLE_OK) return rc;
     auto up = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
-    const size_t plan_off = 0;
+    // the ring comes first: its place does not depend on the count, so its
+    // words hold nothing but statuses of earlier launches
+    const size_t ring_bytes = sizeof(uint64_t) * bsh::batch_ring_words();
+    const size_t plan_off = up(ring_bytes);
     const size_t prefix_off = up(plan_off + sizeof(bsh::BatchPlan) * count);
     const size_t total_off = up(prefix_off + sizeof(uint64_t) * (static_cast<size_t>(count) + 1));
-    const size_t ring_off = up(total_off + sizeof(uint64_t));
-    const size_t need = ring_off + sizeof(uint64_t) * bsh::batch_ring_words();
+    const size_t need = total_off + sizeof(uint64_t);
     {
         std::lock_guard<std::mutex> lock(g_mutex);
         if (ws->aux_bytes < need) {
@@ -530,6 +533,12 @@ int bshuffle_batched(const bshuffle_desc *d_descs, uint32_t count, uint32_t elem
                 ws->aux = nullptr;
                 return cuda_fail(e);
             }
+            e = cudaMemsetAsync(ws->aux, 0, ring_bytes, s);  // tag 0: no status
+            if (e != cudaSuccess) {
+                cudaFree(ws->aux);
+                ws->aux = nullptr;
+                return cuda_fail(e);
+            }
             ws->aux_bytes = bytes;
         }
     }
@@ -539,7 +548,7 @@ int bshuffle_batched(const bshuffle_desc *d_descs, uint32_t count, uint32_t elem
     a.plan = reinterpret_cast<bsh::BatchPlan *>(aux + plan_off);
     a.tile_prefix = reinterpret_cast<uint64_t *>(aux + prefix_off);
     a.total_tiles = reinterpret_cast<uint64_t *>(aux + total_off);
-    a.status = reinterpret_cast<uint64_t *>(aux + ring_off);
+    a.status = reinterpret_cast<uint64_t *>(aux);
     a.count = count;
     a.rounds = rounds;
     a.elem_bytes = elem_bytes;

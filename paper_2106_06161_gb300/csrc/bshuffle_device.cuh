@@ -592,6 +592,13 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 // Waits until every copy group of this thread but the most recent one has landed.
 __device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
+// Waits until every copy group of this thread but the N most recent has landed.
+template <int N>
+__device__ __forceinline__ void cp_async_wait_groups()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 // Barrier 1 over the compute warps only.
 __device__ __forceinline__ void compute_sync(uint32_t threads)
 {

@@ -21,6 +21,8 @@ struct WsHeader {
     uint64_t error_info;  // detail of that error (tile index or slot)
     uint32_t batch_ticket;  // ticket of the persistent batched kernel
     uint32_t batch_done;    // finished CTAs of the persistent batched kernel
+    uint32_t batch_tag;     // first look-back ring tag of the next batched launch
+    uint32_t pad0;
     // Built with BSHUFFLE_LOOKBACK_CLOCKS=1 only: SM clock cycles that tiles
     // waited on the look-back, and cycles the CTAs ran (plain and pipelined
     // single passes); 0 otherwise.
@@ -157,7 +159,7 @@ struct BatchArgs {
     uint64_t timeout_ns;
     int64_t skip_publish_tile;
     WsHeader *ws;
-    uint64_t *status;       // look-back ring of batch_ring_words() words
+    uint64_t *status;       // look-back ring of batch_ring_words() words, tags below ws->batch_tag
     uint64_t *total_tiles;  // written by the planning kernel
 };
 
