@@ -1,4 +1,5 @@
-"""The rounds of domains up to 2^21 run in single precision.
+"""The rounds of domains up to 2^25 run in single precision (from 2^22 with one
+integer multiply-add).
 
 On the CPU: the three fused multiply-adds, in exact integer arithmetic, give
 the words of the 64-bit product for every left half of every width they serve.
@@ -45,8 +46,28 @@ def test_products_exact(L):
     assert np.array_equal(odd & 1, [(w >> (L - 1)) & 1 for w in wide])
 
 
+@pytest.mark.parametrize("L", [11, 12])
+def test_mixed_products_exact(L):
+    left = np.arange(1 << L, dtype=np.int64)
+    mask = (1 << L) - 1
+    wide = [int(v) * M0 for v in left]
+    x = left + TWO23
+    # high word: the pattern of floor(x * 1.694... - its low bits at left = 0), plus left * 1030
+    mul = TWO23 + (LO >> 9)
+    frac = _pattern(x * mul - ((mul & mask) << 23), 23)
+    hi = frac + left * ((HI & 4095) - 1)
+    assert np.array_equal(hi & mask, [(w >> 32) & mask for w in wide])
+    for up in (0, 1):
+        m = -365 << up
+        lo = _pattern(x * m + TWO23 * (1 - m) + (1 << 22), 0)
+        assert np.array_equal(lo & ((2 << L) - 1 if up else mask), [(w & mask) << up if up else w & mask for w in wide])
+    m = LO & mask
+    odd = _pattern(x * m + TWO23 * ((1 << (L - 1)) - m), L - 1)
+    assert np.array_equal(odd & 1, [(w >> (L - 1)) & 1 for w in wide])
+
+
 @pytest.mark.gpu
-@pytest.mark.parametrize("k", range(4, 25))
+@pytest.mark.parametrize("k", range(4, 27))
 def test_indices_match_oracle(k):
     import torch
 
