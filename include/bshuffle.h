@@ -355,12 +355,15 @@ int bshuffle_release_workspaces(void);
  *       while it is resident in L2.  Random HBM accesses are rate-limited on
  *       GB300, streaming ones are not.  Workspace n * (4 + elem_bytes) bytes
  *       plus a little, allocated on first use per stream.  Other n (the
- *       ranked form, bshuffle_permute only): element b's slot is the rank of
+ *       ranked form, bshuffle_permute): element b's slot is the rank of
  *       its domain index i = f^-1(b) among the kept indices (Algorithm 1's
  *       exclusive scan); pass 1 buckets (value, i) by span of domain
  *       indices, a second kernel ranks each span's kept indices with a
  *       bitmap in shared memory, and the window scatter places the values.
  *       Workspace 2^k * (4 + elem_bytes) bytes plus a little.
+ *       bshuffle_inverse of those lengths walks the domain in order instead
+ *       (a look-back gives each chunk's first source slot) and buckets by
+ *       output window; workspace n * (4 + elem_bytes) bytes plus a little.
  *   BSHUFFLE_STRATEGY_PIPELINED  the single pass with its look-back taken
  *       off the compute warps, for gathers and scatters of 4, 8 and 16-byte
  *       elements and for indices (other calls run the plain single pass):
@@ -372,7 +375,8 @@ int bshuffle_release_workspaces(void);
  *   BSHUFFLE_STRATEGY_AUTO (default)  staged when it applies and
  *       n * elem_bytes >= 256 MiB (for n other than 2^k: with 4- or 8-byte
  *       elements only; 16-byte elements run faster on the pipelined single
- *       pass there); otherwise, for n = 2^k >= 16, one launch
+ *       pass there; bshuffle_inverse from 120 MiB on, or from 144 MiB (160 MiB
+ *       with 16-byte elements) where n is under 7/8 of 2^k); otherwise, for n = 2^k >= 16, one launch
  *       without the scan (nothing is dropped, so the i-th domain index is
  *       the i-th kept one: out[i] = in[f(i)], out[f(i)] = in[i] or
  *       out[i] = f(i)); otherwise the pipelined single pass where it applies

@@ -30,7 +30,7 @@ std::atomic<uint64_t> g_timeout_ns{2000000000ull};
 std::atomic<int64_t> g_skip_publish{-1};
 std::atomic<int> g_strategy{BSHUFFLE_STRATEGY_AUTO};
 std::atomic<int> g_pass_timing{0};
-// Auto strategy: the staged path from this many input bytes on.
+// Auto strategy: the staged shuffle from this many input bytes on.
 constexpr uint64_t kStagedMinBytes = uint64_t{1} << 28;
 // Auto strategy: lengths that are not powers of two take the staged path's
 // ranked form for 4- and 8-byte elements (from the same input size), else the
@@ -40,6 +40,24 @@ constexpr uint64_t kStagedMinBytes = uint64_t{1} << 28;
 // 2^28 + 12345 and 2^29 + 3: 4.70 / 9.18 ms against 5.52 / 11.24 ms.  With
 // 16-byte elements the ranked form lost (7.6 against 6.2 ms at 2^28 + 12345).
 bool ranked_by_default(uint32_t elem_bytes) { return elem_bytes == 4 || elem_bytes == 8; }
+// Auto strategy, inverse shuffle: the single-pass scatter's random writes run
+// at the L2's rate while the output fits it (129 MB) and at HBM's, several
+// times slower, beyond; the staged path's time grows with the bytes and, for
+// n < 2^k, with the domain, whose dropped indices its first pass evaluates.
+// So it starts just below the L2's size when little is dropped, and later
+// when up to half is.  Measured on GB300, single pass / staged: 8-byte
+// elements, n near 2^24: 104 MiB 221 / 248 us, 112 MiB 278 / 259, 120 MiB
+// 333 / 273, 2^24 itself 373 / 192; from 2^24 + 1: 128 MiB 401 / 442, 144 MiB
+// 494 / 458, 192 MiB 753 / 504.  4-byte: 112 MiB 437 / 476, 120 MiB 547 / 490,
+// 2^25 + 1 683 / 803, 144 MiB 877 / 830, 256 MiB 2091 / 1027.  16-byte: 120
+// MiB 219 / 218, 2^23 + 1 238 / 284, 160 MiB 324 / 320, 256 MiB 585 / 433.
+bool staged_inverse_by_default(const Geometry &g, uint32_t elem_bytes)
+{
+    constexpr uint64_t kMiB = uint64_t{1} << 20;
+    const uint64_t bytes = uint64_t{g.n} * elem_bytes;
+    if (uint64_t{g.n} * 8 >= g.domain * 7) return bytes >= 120 * kMiB;
+    return bytes >= (elem_bytes == 16 ? 160 : 144) * kMiB;
+}
 // Auto strategy: the pipelined single pass from these domain exponents on.
 // On smaller domains a launch is all latency, and the plain kernel, without
 // the hand-offs between compute warps and look-back warp, finishes first:
@@ -339,8 +357,8 @@ int acquire_staged(cudaStream_t stream, Workspace *ws, size_t bytes)
     return BSHUFFLE_OK;
 }
 
-// The staged path (kernels_staged.cu) for n = 2^k: same output as the fused
-// single pass.  Returns BSHUFFLE_ERR_CUDA without launching anything if its
+// The staged path (kernels_staged.cu): same output as the fused single pass.
+// Returns BSHUFFLE_ERR_CUDA without launching anything if its
 // buffers cannot be allocated.
 int run_staged(const void *in, void *out, uint64_t n, uint32_t elem_bytes, uint64_t seed, uint32_t rounds,
                void *stream_ptr, bool inverse = false)
@@ -350,12 +368,13 @@ int run_staged(const void *in, void *out, uint64_t n, uint32_t elem_bytes, uint6
     a.in = in;
     a.out = out;
     a.g = geometry_of(n);
-    // n < 2^k: the ranked form (gathers only), buckets are spans of domain indices
-    const bool padded = a.g.domain != n;
-    if (padded && inverse) return BSHUFFLE_ERR_INVALID;
+    // the shuffle of n < 2^k: the ranked form, buckets are spans of domain
+    // indices (else windows of output slots)
+    const bool ranked = a.g.domain != n && !inverse;
+    const bool chunked = a.g.domain != n && inverse;  // pass 1 looks back over chunks of the domain
     a.rounds = rounds;
     fill_keys(seed, rounds, a.keys);
-    if (padded) {
+    if (ranked) {
         uint32_t shift = 0, sub = 0;
         bsh::staged_rank_shifts(n, a.g.k, elem_bytes, &shift, &sub);
         a.dst_shift = shift;
@@ -368,8 +387,14 @@ int run_staged(const void *in, void *out, uint64_t n, uint32_t elem_bytes, uint6
         a.num_dst = static_cast<uint32_t>((n + (uint64_t{1} << shift) - 1) >> shift);
     }
 
+    if (chunked) {
+        a.num_tiles = static_cast<uint32_t>(a.g.domain / bsh::staged_p1_tile(n, elem_bytes));
+        a.timeout_ns = g_timeout_ns.load();
+        a.skip_publish_tile = g_skip_publish.load();
+    }
+
     // every bucket reserves its whole span: 2^k entries for the ranked form
-    const uint64_t entries = padded ? a.g.domain : n;
+    const uint64_t entries = ranked ? a.g.domain : n;
     auto up = [](size_t v) { return (v + 255) & ~static_cast<size_t>(255); };
     const size_t off_dval = 0;
     const size_t off_dpos = up(off_dval + entries * elem_bytes);
@@ -378,7 +403,7 @@ int run_staged(const void *in, void *out, uint64_t n, uint32_t elem_bytes, uint6
     const size_t total = up(off_base + a.num_dst * sizeof(uint32_t));
 
     Workspace *ws = nullptr;
-    int rc = acquire_workspace(stream, kMinStatusWords, &ws);
+    int rc = acquire_workspace(stream, chunked ? a.num_tiles : kMinStatusWords, &ws);
     if (rc != BSHUFFLE_OK) return rc;
     rc = acquire_staged(stream, ws, total);
     if (rc != BSHUFFLE_OK) return rc;
@@ -388,6 +413,7 @@ int run_staged(const void *in, void *out, uint64_t n, uint32_t elem_bytes, uint6
     a.dst_cursor = reinterpret_cast<uint32_t *>(base + off_cursor);
     a.bucket_base = reinterpret_cast<uint32_t *>(base + off_base);
     a.ws = ws->header();
+    a.status = ws->status();
     cudaError_t e = cudaMemsetAsync(a.dst_cursor, 0, a.num_dst * sizeof(uint32_t), stream);
     if (e != cudaSuccess) return cuda_fail(e);
     cudaEvent_t *marks = timing_marks(ws);
@@ -405,8 +431,9 @@ bool staged_eligible(uint64_t n, uint32_t elem_bytes)
            (n & (n - 1)) == 0;
 }
 
-// Its ranked form serves the other lengths of the shuffle (not the inverse):
-// the slot of a kept domain index is its rank among the kept indices.
+// The other lengths: the shuffle takes the ranked form (the slot of a kept
+// domain index is its rank among the kept indices), the inverse a pass 1 over
+// the domain with a look-back.
 bool ranked_eligible(uint64_t n, uint32_t elem_bytes)
 {
     return (elem_bytes == 4 || elem_bytes == 8 || elem_bytes == 16) && n >= 2 * bsh::staged_tile_size() &&
@@ -470,7 +497,8 @@ int bshuffle_inverse(const void *in, void *out, uint64_t n, uint32_t elem_bytes,
     if (rc != BSHUFFLE_OK) return rc;
     const int strategy = g_strategy.load();
     if ((strategy == BSHUFFLE_STRATEGY_AUTO || strategy == BSHUFFLE_STRATEGY_STAGED) &&
-        staged_eligible(n, elem_bytes) && (strategy == BSHUFFLE_STRATEGY_STAGED || n * elem_bytes >= kStagedMinBytes)) {
+        (staged_eligible(n, elem_bytes) || ranked_eligible(n, elem_bytes)) &&
+        (strategy == BSHUFFLE_STRATEGY_STAGED || staged_inverse_by_default(geometry_of(n), elem_bytes))) {
         rc = run_staged(in, out, n, elem_bytes, seed, rounds, stream, true);
         if (rc == BSHUFFLE_OK || strategy == BSHUFFLE_STRATEGY_STAGED) return rc;
         // auto: the staged buffers could not be had; the single pass needs none

@@ -486,13 +486,12 @@ struct TileShared {
 };
 
 // Run by one full warp after every warp has written its counts: exclusive
-// scan of the ENTRIES counts in place, publication of the tile aggregate,
-// look-back, publication of the inclusive prefix.  Publishing is skipped for
-// the tile `skip_tile` (test hook).
+// scan of the ENTRIES counts in place and publication of the tile aggregate,
+// which is returned.  Publishing is skipped for the tile `skip_tile` (test
+// hook).
 template <int ENTRIES>
-__device__ __forceinline__ void tile_scan_lookback(TileShared<ENTRIES> &st, const StatusRing &ring, uint64_t tile,
-                                                   uint64_t first, uint64_t timeout_ns, int64_t skip_tile,
-                                                   WsHeader *ws)
+__device__ __forceinline__ uint32_t tile_scan_publish(TileShared<ENTRIES> &st, const StatusRing &ring, uint64_t tile,
+                                                      uint64_t first, int64_t skip_tile)
 {
     constexpr int C = (ENTRIES + 31) / 32;
     const uint32_t lane = threadIdx.x & 31u;
@@ -513,16 +512,27 @@ __device__ __forceinline__ void tile_scan_lookback(TileShared<ENTRIES> &st, cons
         run += local[c];
     }
     const uint32_t aggregate = __shfl_sync(kFull, incl, 31);
+    if (lane == 0 && static_cast<int64_t>(tile) != skip_tile)
+        st_relaxed_gpu(ring.slot(tile), status_word(ring.tag(tile), tile == first, aggregate));
+    return aggregate;
+}
+
+// Then, by the same warp: look-back and publication of the inclusive prefix.
+template <int ENTRIES>
+__device__ __forceinline__ void tile_lookback(TileShared<ENTRIES> &st, uint32_t aggregate, const StatusRing &ring,
+                                              uint64_t tile, uint64_t first, uint64_t timeout_ns, int64_t skip_tile,
+                                              WsHeader *ws)
+{
+    const uint32_t lane = threadIdx.x & 31u;
     const bool publish = static_cast<int64_t>(tile) != skip_tile;
-    const uint32_t tag = ring.tag(tile);
-    if (lane == 0 && publish) st_relaxed_gpu(ring.slot(tile), status_word(tag, tile == first, aggregate));
     uint32_t exclusive = 0;
     bool ok = true;
     if (tile > first) {
         const long long c0 = clock_mark();
         exclusive = lookback(ring, tile, first, timeout_ns, ok);
         if (lane == 0) clock_add(&ws->lookback_cycles, c0);
-        if (lane == 0 && publish) st_relaxed_gpu(ring.slot(tile), status_word(tag, true, exclusive + aggregate));
+        if (lane == 0 && publish)
+            st_relaxed_gpu(ring.slot(tile), status_word(ring.tag(tile), true, exclusive + aggregate));
         if (lane == 0 && !ok) record_error(ws, kErrLookbackTimeout, tile);
     }
     if (lane == 0) {
@@ -530,6 +540,16 @@ __device__ __forceinline__ void tile_scan_lookback(TileShared<ENTRIES> &st, cons
         st.aggregate = aggregate;
         st.ok = ok ? 1u : 0u;
     }
+}
+
+// Both steps at once.
+template <int ENTRIES>
+__device__ __forceinline__ void tile_scan_lookback(TileShared<ENTRIES> &st, const StatusRing &ring, uint64_t tile,
+                                                   uint64_t first, uint64_t timeout_ns, int64_t skip_tile,
+                                                   WsHeader *ws)
+{
+    const uint32_t aggregate = tile_scan_publish(st, ring, tile, first, skip_tile);
+    tile_lookback(st, aggregate, ring, tile, first, timeout_ns, skip_tile, ws);
 }
 
 // Called by one thread per CTA once the CTA no longer reads the header: the

@@ -177,9 +177,10 @@ cudaError_t launch_batched(const BatchArgs &a, cudaStream_t stream);
 // ------------------------------------------------------------------ staged path
 
 // The staged shuffle: same output as the fused single pass, two streaming
-// passes (see kernels_staged.cu).  For n == 2^k a bucket is a window of
-// output slots; for other n (the ranked form) a bucket is a window of domain
-// indices, and the second pass ranks its kept indices with a bitmap.
+// passes (see kernels_staged.cu).  For n == 2^k and for the inverse shuffle a
+// bucket is a window of output slots; for the shuffle of other n (the ranked
+// form) a bucket is a window of domain indices, and the second pass ranks its
+// kept indices with a bitmap.
 struct StagedArgs {
     const void *in;
     void *out;
@@ -192,11 +193,18 @@ struct StagedArgs {
     uint32_t *dpos;         // offsets within the bucket's span
     uint32_t *dst_cursor;   // num_dst, zero at launch
     uint32_t *bucket_base;  // ranked: num_dst first slots, written by pass 2a
-    WsHeader *ws;           // error word
+    WsHeader *ws;           // error word; inverse of n < 2^k: also its tickets
+    uint64_t *status;       // inverse of n < 2^k: one look-back word per chunk
+    uint32_t num_tiles;     // inverse of n < 2^k: chunks of staged_p1_tile() domain indices
+    uint32_t pad0;
+    uint64_t timeout_ns;
+    int64_t skip_publish_tile;
     uint32_t keys[kMaxRounds];
 };
 
 uint32_t staged_tile_size();
+// Elements (inverse of n < 2^k: domain indices) per chunk of pass 1.
+uint32_t staged_p1_tile(uint64_t n, uint32_t elem_bytes);
 // log2 of the destination bucket (output window) in elements for a staged
 // shuffle of n = 2^k elements of elem_bytes.
 uint32_t staged_window_shift(uint64_t n, uint32_t elem_bytes);

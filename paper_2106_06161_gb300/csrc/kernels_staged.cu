@@ -25,6 +25,11 @@
 // by its exact slot, so the output is deterministic and identical to the
 // single pass.
 //
+// The inverse shuffle of those lengths needs no rank per entry: its P1 walks
+// the domain in order, so the source slot of a kept index is the running count
+// of Algorithm 1's scan (decoupled look-back over the chunks), and its target
+// is the image itself: windows of output slots and P2 as for n = 2^k.
+//
 // Sizes (measured on GB300): P2 is fastest in small windows (its random
 // writes stay in L2; 4 MiB beats 8 MiB by 13 %, 32 MiB costs 50 % more), while
 // P1 slows down steeply past 256 buckets per 2,048-element chunk (each chunk
@@ -219,6 +224,132 @@ __global__ void __launch_bounds__(kP1Block, BSHUFFLE_RANKED_P1_MIN_CTAS)
     bucket_pass<T, ODD, false, 16, true>(a);
 }
 
+// The inverse shuffle's P1 for n < 2^k: out[f(i_j)] = in[j].  A CTA owns a
+// chunk of consecutive domain indices (a ticket, so that its predecessors are
+// running), evaluates the bijection forward, publishes its kept count, and
+// looks back for the rank of its first kept index while it counts its images
+// by output window; the source slots of its kept indices are then consecutive,
+// so their elements are read coalesced, sorted by window in shared memory and
+// appended as in bucket_pass.  Every window of 2^dst_shift output slots gets
+// exactly one entry per slot.
+// The single-pass scatter that it replaces above the L2's size is bound by
+// random writes to HBM.  Measured on GB300, single pass and staged: uint64 at
+// 2^25 + 1 1.10 and 0.84 ms, 2^26 + 1 2.49 and 1.86, 2^27 - 5 5.17 and 2.45;
+// uint32 at 2^26 - 5 2.09 and 1.03; 16-byte at 2^25 - 7 1.28 and 0.91.  This
+// pass is bound by the cipher over the whole domain (the odd-k forward round)
+// and waits on the look-back: publishing the count before the window counts
+// took 2^28 + 12345 uint64 from 8.93 to 8.65 ms (single pass 10.7).
+template <class T, bool ODD, int ITEMS>
+__global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const __grid_constant__ StagedArgs a)
+{
+    constexpr uint32_t kTile = kP1Block * ITEMS;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    T *s_val = reinterpret_cast<T *>(s_raw);
+    uint32_t *s_dst = reinterpret_cast<uint32_t *>(s_raw + kTile * sizeof(T));
+    uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_raw + kTile * (sizeof(T) + 4));
+    uint32_t *s_start = s_cnt + a.num_dst;
+    uint32_t *s_gbase = s_start + a.num_dst;
+    __shared__ dev::TileShared<ITEMS * kP1Warps> st;
+    __shared__ uint32_t s_warp[kP1Warps];
+
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const Geometry &g = a.g;
+    if (tid == 0) {
+        st.tile = atomicAdd(&a.ws->ticket, 1u);
+        st.tag = dev::ld_relaxed_gpu(&a.ws->tag);
+    }
+    for (uint32_t q = tid; q < a.num_dst; q += kP1Block) s_cnt[q] = 0u;
+    __syncthreads();
+    const uint32_t tile = st.tile, tag = st.tag;
+    if (tile >= a.num_tiles) {  // only a corrupted header could hand out such a ticket
+        if (tid == 0) {
+            dev::record_error(a.ws, dev::kErrDeviceBounds, tile);
+            dev::finish_launch(a.ws, tag, gridDim.x);
+        }
+        return;
+    }
+    // the domain is a multiple of the chunk
+    const uint32_t base = tile * kTile + tid;
+    uint32_t left[ITEMS], right[ITEMS];
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t i = base + static_cast<uint32_t>(j * kP1Block);
+        left[j] = i >> g.R;
+        right[j] = i & g.rmask;
+    }
+    dev::cipher_items<ODD, ITEMS>(left, right, a.keys, a.rounds, g);
+    uint32_t dst[ITEMS], mask[ITEMS], slot[ITEMS];
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        dst[j] = (left[j] << g.R) | right[j];
+        mask[j] = __ballot_sync(kFull, dst[j] < g.n);
+        if (lane == 0) st.counts[j * kP1Warps + warp] = static_cast<uint32_t>(__popc(mask[j]));
+    }
+    __syncthreads();
+    // the last warp publishes the chunk's count before anything else: later
+    // chunks wait for it
+    const bool ranker = warp == kP1Warps - 1;
+    const dev::StatusRing ring{a.status, ~0ull, 63u, tag};
+    uint32_t aggregate = 0;
+    if (ranker) aggregate = dev::tile_scan_publish(st, ring, tile, 0, a.skip_publish_tile);
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j)
+        if (dst[j] < g.n) slot[j] = atomicAdd(&s_cnt[dst[j] >> a.dst_shift], 1u);
+    __syncthreads();
+    // and looks back while the others append the window counts
+    if (ranker) {
+        dev::tile_lookback(st, aggregate, ring, tile, 0, a.timeout_ns, a.skip_publish_tile, a.ws);
+    } else {
+        for (uint32_t q = tid; q < a.num_dst; q += kP1Block - 32u) {
+            const uint32_t c = s_cnt[q];
+            s_gbase[q] = c != 0u ? atomicAdd(&a.dst_cursor[q], c) : 0u;
+        }
+    }
+    block_exclusive_scan(s_cnt, s_start, a.num_dst, s_warp);
+    __syncthreads();
+    // an unranked chunk (the look-back ran out of time) moves zeros: its
+    // window entries have to be there for the next pass
+    const bool ok = st.ok != 0u;
+    const uint32_t prefix = st.prefix, lt = dev::lanemask_lt();
+    const T *in = static_cast<const T *>(a.in);
+    T val[ITEMS];
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        val[j] = T{};
+        if (dst[j] >= g.n) continue;
+        const uint32_t src = prefix + st.counts[j * kP1Warps + warp] + static_cast<uint32_t>(__popc(mask[j] & lt));
+        if (ok && src < g.n) val[j] = __ldcs(in + src);
+        else if (ok) dev::record_error(a.ws, dev::kErrDeviceBounds, src);
+    }
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        if (dst[j] >= g.n) continue;
+        const uint32_t p = s_start[dst[j] >> a.dst_shift] + slot[j];
+        s_val[p] = val[j];
+        s_dst[p] = dst[j];
+    }
+    __syncthreads();
+    T *dval = static_cast<T *>(a.dval);
+    const uint32_t bmask = (1u << a.dst_shift) - 1u;
+    const uint32_t kept = st.aggregate;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t p = static_cast<uint32_t>(j * kP1Block) + tid;
+        if (p >= kept) continue;
+        const uint32_t d = s_dst[p];
+        const uint32_t q = d >> a.dst_shift;
+        const uint32_t off = s_gbase[q] + (p - s_start[q]);
+        const uint64_t o = (static_cast<uint64_t>(q) << a.dst_shift) + off;
+        if (off <= bmask && o < g.n) {
+            dval[o] = s_val[p];
+            a.dpos[o] = d & bmask;
+        } else {
+            dev::record_error(a.ws, dev::kErrDeviceBounds, o);
+        }
+    }
+    if (tid == 0) dev::finish_launch(a.ws, tag, gridDim.x);
+}
+
 // ------------------------------------------------------------------ P2
 
 // P2: each thread moves kSItems entries (reads first, then the stores).
@@ -229,10 +360,12 @@ __global__ void __launch_bounds__(kP1Block, BSHUFFLE_RANKED_P1_MIN_CTAS)
 constexpr int kScatterCtasPerSm = 5;
 constexpr size_t kScatterSmemReserve = (228u * 1024u) / kScatterCtasPerSm - 1024u;
 
-template <class T>
+// RAGGED: n < 2^k, whose last chunk is not full (the entries of the windows
+// are n in a row, since every window but the last one is).
+template <class T, bool RAGGED>
 __global__ void __launch_bounds__(kSBlock) staged_scatter_kernel(const __grid_constant__ StagedArgs a)
 {
-    const uint32_t n = a.g.n;  // n = 2^k <= 2^31, a multiple of kSTile
+    const uint32_t n = a.g.n;  // not RAGGED: n = 2^k <= 2^31, a multiple of kSTile
     const uint32_t first = blockIdx.x * kSTile;
     const T *dval = static_cast<const T *>(a.dval);
     T *out = static_cast<T *>(a.out);
@@ -241,11 +374,13 @@ __global__ void __launch_bounds__(kSBlock) staged_scatter_kernel(const __grid_co
 #pragma unroll
     for (int j = 0; j < kSItems; ++j) {
         const uint32_t e = first + static_cast<uint32_t>(j * kSBlock) + threadIdx.x;
+        if (RAGGED && e - first >= n - first) continue;
         v[j] = __ldcs(dval + e);
         dst[j] = ((e >> a.dst_shift) << a.dst_shift) + __ldcs(a.dpos + e);
     }
 #pragma unroll
     for (int j = 0; j < kSItems; ++j) {
+        if (RAGGED && static_cast<uint32_t>(j * kSBlock) + threadIdx.x >= n - first) continue;
         if (dst[j] < n) out[dst[j]] = v[j];
         else dev::record_error(a.ws, dev::kErrDeviceBounds, dst[j]);
     }
@@ -564,6 +699,23 @@ cudaError_t launch_rank(const StagedArgs &a, int device, cudaStream_t stream)
 }
 
 
+// P1 of the inverse shuffle for n < 2^k.
+template <class T, int ITEMS>
+cudaError_t launch_inverse_p1(const StagedArgs &a, int device, cudaStream_t stream)
+{
+    const auto odd = staged_inverse_bucket_kernel<T, true, ITEMS>, even = staged_inverse_bucket_kernel<T, false, ITEMS>;
+    static std::atomic<bool> configured[64];  // attribute set on this device
+    if (!configured[device].load(std::memory_order_acquire)) {
+        const int most = static_cast<int>(p1_smem_bytes<T, ITEMS>(4096));
+        cudaError_t e = cudaFuncSetAttribute(odd, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(even, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e != cudaSuccess) return e;
+        configured[device].store(true, std::memory_order_release);
+    }
+    ((a.g.k & 1u) ? odd : even)<<<a.num_tiles, kP1Block, p1_smem_bytes<T, ITEMS>(a.num_dst), stream>>>(a);
+    return cudaGetLastError();
+}
+
 template <class T, bool FORWARD>
 cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t stream, cudaEvent_t *marks)
 {
@@ -573,8 +725,11 @@ cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t strea
     if (e != cudaSuccess) return e;
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
     if (!configured[device].load(std::memory_order_acquire)) {
-        e = cudaFuncSetAttribute(staged_scatter_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(staged_scatter_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(kScatterSmemReserve));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(staged_scatter_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     static_cast<int>(kScatterSmemReserve));
         if (e != cudaSuccess) return e;
         configured[device].store(true, std::memory_order_release);
     }
@@ -585,8 +740,10 @@ cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t strea
         if constexpr (!FORWARD)
             e = items == 16 ? launch_p1<T, false, 16, true>(a, device, stream)
                             : launch_p1<T, false, 8, true>(a, device, stream);
+        else if constexpr (sizeof(T) <= 8)
+            e = items == 16 ? launch_inverse_p1<T, 16>(a, device, stream) : launch_inverse_p1<T, 8>(a, device, stream);
         else
-            e = cudaErrorInvalidValue;  // the inverse shuffle has no ranked form
+            e = launch_inverse_p1<T, 8>(a, device, stream);
     } else if constexpr (sizeof(T) <= 8) {
         e = items == 16 ? launch_p1<T, FORWARD, 16, false>(a, device, stream)
                         : launch_p1<T, FORWARD, 8, false>(a, device, stream);
@@ -595,11 +752,14 @@ cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t strea
     }
     if (e == cudaSuccess) e = mark(marks, 1, stream);
     if (e != cudaSuccess) return e;
-    if (padded) {
+    const unsigned chunks = static_cast<unsigned>((static_cast<uint64_t>(a.g.n) + kSTile - 1) / kSTile);
+    if (padded && !FORWARD) {
         e = launch_rank<T>(a, device, stream);
+    } else if (padded) {
+        staged_scatter_kernel<T, true><<<chunks, kSBlock, kScatterSmemReserve, stream>>>(a);
+        e = cudaGetLastError();
     } else {
-        const unsigned chunks = static_cast<unsigned>(static_cast<uint64_t>(a.g.n) / kSTile);
-        staged_scatter_kernel<T><<<chunks, kSBlock, kScatterSmemReserve, stream>>>(a);
+        staged_scatter_kernel<T, false><<<chunks, kSBlock, kScatterSmemReserve, stream>>>(a);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = mark(marks, 2, stream);
@@ -631,6 +791,11 @@ void rank_config(uint64_t n, uint32_t k, uint32_t elem_bytes, uint32_t *bucket_s
 
 uint32_t staged_tile_size() { return kStagedMinChunk; }
 
+uint32_t staged_p1_tile(uint64_t n, uint32_t elem_bytes)
+{
+    return p1_items_for(n, elem_bytes) == 16u ? kP1TileLarge : kP1TileSmall;
+}
+
 uint32_t staged_window_shift(uint64_t n, uint32_t elem_bytes)
 {
     uint32_t lg = 0;
@@ -660,11 +825,16 @@ cudaError_t launch_staged(const StagedArgs &a, uint32_t elem_bytes, bool inverse
 {
     uint32_t items = p1_items_for(a.g.n, elem_bytes);
     const uint64_t p1_tile = items == 16 ? kP1TileLarge : kP1TileSmall;
-    if (static_cast<uint64_t>(a.g.n) != a.g.domain) {
-        // ranked form: any n below its 2^k domain, gathers only
+    if (static_cast<uint64_t>(a.g.n) != a.g.domain && inverse) {
+        if (a.num_dst > 4096 || a.g.domain < 2 * kStagedMinChunk || a.g.domain > (uint64_t{1} << 32) ||
+            a.g.domain != uint64_t{a.num_tiles} * p1_tile || a.dst_shift >= 32u ||
+            a.num_dst != ((uint64_t{a.g.n} + (uint64_t{1} << a.dst_shift) - 1) >> a.dst_shift))
+            return cudaErrorInvalidValue;
+    } else if (static_cast<uint64_t>(a.g.n) != a.g.domain) {
+        // ranked form: any n below its 2^k domain
         uint32_t s = 0, w = 0;
         rank_config(a.g.n, a.g.k, elem_bytes, &s, &w, &items);
-        if (inverse || a.g.n == 0 || a.g.domain > (uint64_t{1} << 32) || a.dst_shift != s || a.sub_shift != w ||
+        if (a.g.n == 0 || a.g.domain > (uint64_t{1} << 32) || a.dst_shift != s || a.sub_shift != w ||
             (static_cast<uint64_t>(a.num_dst) << a.dst_shift) != a.g.domain || a.num_dst > 4096)
             return cudaErrorInvalidValue;
     } else if (a.num_dst > 4096 || a.g.domain < 2 * kStagedMinChunk || a.g.domain > (uint64_t{1} << 31) ||
