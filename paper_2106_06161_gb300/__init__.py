@@ -77,8 +77,14 @@ __all__ = [
 ]
 
 
+# The current stream's handle, without the Stream object around it (2.1 us of
+# a small call against 0.2).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 def _stream_of(t: torch.Tensor) -> int:
-    return torch.cuda.current_stream(t.device).cuda_stream
+    return _raw_stream(t.get_device())
 
 
 def _require_cuda(t: torch.Tensor, what: str) -> None:
@@ -90,6 +96,8 @@ def _require_cuda(t: torch.Tensor, what: str) -> None:
 
 def row_bytes(t: torch.Tensor) -> int:
     """Bytes of one element along dim 0 (a scalar or a whole row)."""
+    if t.dim() == 1:
+        return t.element_size()
     per = 1
     for s in t.shape[1:]:
         per *= s
@@ -104,26 +112,26 @@ def _out_like(x: torch.Tensor, out: torch.Tensor | None) -> torch.Tensor:
     return out
 
 
-def _along(fn, x: torch.Tensor, seed: int, rounds: int, out, dim: int) -> torch.Tensor:
+def _rows0(call, x: torch.Tensor, seed: int, rounds: int, out) -> torch.Tensor:
+    """One shuffle (or its inverse) of a CUDA tensor along dim 0."""
+    x = x.contiguous()
+    out = _out_like(x, out)
+    call(x.data_ptr(), out.data_ptr(), x.size(0), row_bytes(x), seed, rounds, _stream_of(x))
+    return out
+
+
+def _along(call, x: torch.Tensor, seed: int, rounds: int, out, dim: int) -> torch.Tensor:
     """Apply a dim-0 call along `dim`: the dimension is moved to the front (a
     copy), its slices are shuffled as rows, and it is moved back (a copy)."""
-    d = dim % x.dim() if x.dim() else 0
+    d = dim % x.dim()
     if d == 0:
-        return fn(x, seed, rounds, out)
-    y = fn(x.movedim(d, 0).contiguous(), seed, rounds, None).movedim(0, d)
+        return _rows0(call, x, seed, rounds, out)
+    y = _rows0(call, x.movedim(d, 0), seed, rounds, None).movedim(0, d)
     if out is None:
         return y.contiguous()
     if out.shape != x.shape or out.dtype != x.dtype or out.device != x.device:
         raise ValueError("out must have the input's shape, dtype and device")
     return out.copy_(y)
-
-
-def _permute0(x: torch.Tensor, seed: int, rounds: int, out) -> torch.Tensor:
-    _require_cuda(x, "x")
-    x = x.contiguous()
-    out = _out_like(x, out)
-    bshuffle_permute(x.data_ptr(), out.data_ptr(), x.shape[0], row_bytes(x), seed, rounds, _stream_of(x))
-    return out
 
 
 def permute(x: torch.Tensor, seed: int, rounds: int = DEFAULT_ROUNDS,
@@ -132,22 +140,14 @@ def permute(x: torch.Tensor, seed: int, rounds: int = DEFAULT_ROUNDS,
     j and i_j indexing that dimension.  The slices along `dim` are the
     elements shuffled: 1, 2, 4 or 8 bytes, or a multiple of 16 bytes."""
     _require_cuda(x, "x")
-    return _along(_permute0, x, seed, rounds, out, dim)
-
-
-def _inverse0(y: torch.Tensor, seed: int, rounds: int, out) -> torch.Tensor:
-    _require_cuda(y, "y")
-    y = y.contiguous()
-    out = _out_like(y, out)
-    bshuffle_inverse(y.data_ptr(), out.data_ptr(), y.shape[0], row_bytes(y), seed, rounds, _stream_of(y))
-    return out
+    return _along(bshuffle_permute, x, seed, rounds, out, dim)
 
 
 def inverse(y: torch.Tensor, seed: int, rounds: int = DEFAULT_ROUNDS,
             out: torch.Tensor | None = None, dim: int = 0) -> torch.Tensor:
     """Undo :func:`permute` along `dim`: out[f(i_j)] = y[j]."""
     _require_cuda(y, "y")
-    return _along(_inverse0, y, seed, rounds, out, dim)
+    return _along(bshuffle_inverse, y, seed, rounds, out, dim)
 
 
 def indices(n: int, seed: int, rounds: int = DEFAULT_ROUNDS, dtype: torch.dtype = torch.int64,
@@ -165,12 +165,30 @@ def indices(n: int, seed: int, rounds: int = DEFAULT_ROUNDS, dtype: torch.dtype 
 
 def _descs(in_ptrs, out_ptrs, sizes, seeds, device) -> torch.Tensor:
     """Device array of bshuffle_desc {in, out, n, seed} as int64 words."""
-    host = np.empty((len(sizes), 4), dtype=np.uint64)
+    # Pinned memory is copied in stream order, so that the host does not wait
+    # for the work already on the stream; it goes back to PyTorch's pool, which
+    # keeps it until the copy is done.  A stream under capture refuses the copy
+    # of pageable memory: a graph must not read this buffer again.
+    pinned = not torch.cuda.is_current_stream_capturing()
+    words = torch.empty((len(sizes), 4), dtype=torch.int64, pin_memory=pinned)
+    host = words.numpy().view(np.uint64)
     host[:, 0] = np.asarray(in_ptrs, dtype=np.uint64)
     host[:, 1] = np.asarray(out_ptrs, dtype=np.uint64)
     host[:, 2] = np.asarray(sizes, dtype=np.uint64)
-    host[:, 3] = np.asarray([s & (2**64 - 1) for s in seeds], dtype=np.uint64)
-    return torch.from_numpy(host.view(np.int64)).to(device, non_blocking=False)
+    host[:, 3] = _seed_words(seeds)
+    return words.to(device, non_blocking=pinned)
+
+
+def _seed_words(seeds: list) -> np.ndarray:
+    """The seeds modulo 2^64."""
+    if set(map(type, seeds)) <= {int}:
+        try:
+            words = np.asarray(seeds)
+            if words.dtype in (np.int64, np.uint64):
+                return words.view(np.uint64)
+        except OverflowError:
+            pass
+    return np.asarray([s & (2**64 - 1) for s in seeds], dtype=np.uint64)
 
 
 def batched(inputs: list[torch.Tensor], seeds, rounds: int = DEFAULT_ROUNDS,

@@ -103,6 +103,8 @@ class BShuffleError(RuntimeError):
 def load() -> ctypes.CDLL:
     """Load the in-tree libbshuffle.so (built by paper_2106_06161_gb300.build)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):

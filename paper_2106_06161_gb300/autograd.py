@@ -10,20 +10,20 @@ from __future__ import annotations
 
 import torch
 
+from . import inverse, permute
+
 
 class BShuffleRows(torch.autograd.Function):
     """y = x[indices(len(x), seed, rounds)] with a scatter backward."""
 
     @staticmethod
     def forward(ctx, x: torch.Tensor, seed: int, rounds: int):
-        from . import permute
         ctx.seed = seed
         ctx.rounds = rounds
         return permute(x, seed, rounds)
 
     @staticmethod
     def backward(ctx, grad_out: torch.Tensor):
-        from . import inverse
         return inverse(grad_out.contiguous(), ctx.seed, ctx.rounds), None, None
 
 
