@@ -375,9 +375,10 @@ int bshuffle_release_workspaces(void);
  *   BSHUFFLE_STRATEGY_AUTO (default)  staged when it applies and
  *       n * elem_bytes >= 256 MiB (for n other than 2^k: with 4- or 8-byte
  *       elements only; 16-byte elements run faster on the pipelined single
- *       pass there; bshuffle_inverse from 120 MiB on, or from 144 MiB (160 MiB
- *       with 16-byte elements) where n is under 7/8 of 2^k); otherwise, for n = 2^k >= 16, one launch
- *       without the scan (nothing is dropped, so the i-th domain index is
+ *       pass there; bshuffle_inverse of other n also from 126 MiB on where n
+ *       is at least 3/4 of 2^k, with 16-byte elements only there and from 224
+ *       MiB on, and of n = 2^k with 4- or 8-byte elements from 128 MiB on);
+ *       otherwise, for n = 2^k >= 16, one launch without the scan (nothing is dropped, so the i-th domain index is
  *       the i-th kept one: out[i] = in[f(i)], out[f(i)] = in[i] or
  *       out[i] = f(i)); otherwise the pipelined single pass where it applies
  *       and the domain has at least 2^18 indices (2^19 for the scatter of

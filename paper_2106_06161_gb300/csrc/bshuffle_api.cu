@@ -44,19 +44,23 @@ bool ranked_by_default(uint32_t elem_bytes) { return elem_bytes == 4 || elem_byt
 // at the L2's rate while the output fits it (129 MB) and at HBM's, several
 // times slower, beyond; the staged path's time grows with the bytes and, for
 // n < 2^k, with the domain, whose dropped indices its first pass evaluates.
-// So it starts just below the L2's size when little is dropped, and later
-// when up to half is.  Measured on GB300, single pass / staged: 8-byte
-// elements, n near 2^24: 104 MiB 221 / 248 us, 112 MiB 278 / 259, 120 MiB
-// 333 / 273, 2^24 itself 373 / 192; from 2^24 + 1: 128 MiB 401 / 442, 144 MiB
-// 494 / 458, 192 MiB 753 / 504.  4-byte: 112 MiB 437 / 476, 120 MiB 547 / 490,
-// 2^25 + 1 683 / 803, 144 MiB 877 / 830, 256 MiB 2091 / 1027.  16-byte: 120
-// MiB 219 / 218, 2^23 + 1 238 / 284, 160 MiB 324 / 320, 256 MiB 585 / 433.
+// The lines lie where the staged path wins on every GB300 measured (the random
+// writes of some are a quarter faster than of others).  Single pass on a
+// slower and a faster one / staged, us: 8-byte elements at 2^24 - 5 312 and
+// 301 / 273, 3 2^23 + 1 735 and 605 / 518, 2^24 + 1 334 and 328 / 442, 2^25 + 1
+// 1085 and 864 / 849; 4-byte at 2^25 - 5 562 and 543 / 499, 3 2^24 + 1 1391 and
+// 1139 / 922, 2^25 + 1 579 and 576 / 597; 16-byte at 2^23 - 5 192 and 184 /
+// 227, 2^24 - 5 578 and 457 / 428, 2^24 + 1 583 and 465 / 591.  n = 2^k, where
+// nothing is ranked: 8-byte at 2^24 312 / 191, 4-byte at 2^25 535 / 397,
+// 16-byte at 2^23 176 / 170, 8-byte at 2^23 52 / 111.
 bool staged_inverse_by_default(const Geometry &g, uint32_t elem_bytes)
 {
     constexpr uint64_t kMiB = uint64_t{1} << 20;
-    const uint64_t bytes = uint64_t{g.n} * elem_bytes;
-    if (uint64_t{g.n} * 8 >= g.domain * 7) return bytes >= 120 * kMiB;
-    return bytes >= (elem_bytes == 16 ? 160 : 144) * kMiB;
+    const uint64_t n = g.n, bytes = n * elem_bytes;
+    if (n == g.domain) return bytes >= (elem_bytes == 16 ? kStagedMinBytes : 128 * kMiB);
+    const bool mostly_kept = n * 4 >= g.domain * 3;
+    if (elem_bytes == 16) return mostly_kept && bytes >= 224 * kMiB;
+    return bytes >= kStagedMinBytes || (mostly_kept && bytes >= 126 * kMiB);
 }
 // Auto strategy: the pipelined single pass from these domain exponents on.
 // On smaller domains a launch is all latency, and the plain kernel, without
@@ -299,7 +303,7 @@ int run_fused(const void *in, void *out, uint64_t n, uint32_t elem_bytes, uint64
     const int config = rows ? 0 : bsh::elem_config_for(elem_bytes, mode, rounds);
     const int pipe_config = pipe ? bsh::pipe_config_for(elem_bytes, mode) : 0;
     const uint64_t tile = rows   ? bsh::rows_tile_size(elem_bytes)
-                          : pipe ? bsh::pipe_tile_size(elem_bytes, pipe_config)
+                          : pipe ? bsh::pipe_tile_size(elem_bytes, pipe_config, mode, a.g.k)
                                  : bsh::elem_tile_size(config);
     const uint64_t tiles = (a.g.domain + tile - 1) / tile;
     a.num_tiles = static_cast<uint32_t>(tiles);

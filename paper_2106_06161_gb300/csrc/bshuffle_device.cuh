@@ -568,8 +568,8 @@ __device__ __forceinline__ void finish_launch(WsHeader *ws, uint32_t tag, uint32
 }
 
 // ------------------------------------------------------------------ async copies and mbarriers
-// Helpers of the pipelined kernels: shared-memory mbarriers, cp.async copies
-// global -> shared, and a named barrier over a subset of the CTA's warps.
+// Helpers of the pipelined kernels: shared-memory mbarriers and cp.async copies
+// global -> shared.
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
@@ -647,12 +647,6 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait_groups()
 {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// Barrier 1 over the compute warps only.
-__device__ __forceinline__ void compute_sync(uint32_t threads)
-{
-    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
 }
 
 }  // namespace dev

@@ -279,7 +279,7 @@ int pipe_config_for(uint32_t elem_bytes, Mode mode);
 int select_pipe_config(uint32_t elem_bytes, int config);
 int selected_pipe_config(uint32_t elem_bytes);
 bool pipe_supports(Mode mode, uint32_t elem_bytes);
-uint32_t pipe_tile_size(uint32_t elem_bytes, int config);
+uint32_t pipe_tile_size(uint32_t elem_bytes, int config, Mode mode, uint32_t k);
 cudaError_t launch_pipe(const TileArgs &a, Mode mode, uint32_t elem_bytes, int config, cudaStream_t stream);
 cudaError_t launch_pipe_tuned(const TileArgs &a, uint32_t elem_bytes, int config, cudaStream_t stream);
 

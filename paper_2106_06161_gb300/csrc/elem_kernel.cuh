@@ -37,12 +37,6 @@ using dev::kFull;
 
 enum Bijection : int { kVarPhilox = 0, kLcg = 1 };
 
-template <class T>
-__device__ __forceinline__ T load_nc(const T *p)
-{
-    return __ldg(p);
-}
-
 template <class T, Mode MODE, bool ODD, int BLOCK, int ITEMS, int ROUNDS, int BIJ = kVarPhilox, bool RANGE = false>
 __global__ void __launch_bounds__(BLOCK) elem_tile_kernel(const __grid_constant__ TileArgs a)
 {
@@ -110,7 +104,7 @@ __global__ void __launch_bounds__(BLOCK) elem_tile_kernel(const __grid_constant_
         const T *in = static_cast<const T *>(a.in);
 #pragma unroll
         for (int j = 0; j < ITEMS; ++j)
-            if (keep[j]) val[j] = load_nc(in + src[j]);
+            if (keep[j]) val[j] = __ldg(in + src[j]);
     }
 
     // 3. in-tile ranks and the tile's global prefix
@@ -160,7 +154,7 @@ __global__ void __launch_bounds__(BLOCK) elem_tile_kernel(const __grid_constant_
             T *out = static_cast<T *>(a.out);
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
-                if (keep[j]) val[j] = load_nc(in + dst[j]);
+                if (keep[j]) val[j] = __ldcs(in + dst[j]);
 #pragma unroll
             for (int j = 0; j < ITEMS; ++j)
                 if (keep[j]) out[src[j]] = val[j];

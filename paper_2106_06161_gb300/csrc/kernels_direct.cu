@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kDBlock) direct_elem_kernel(const __grid_const
         T v[kDItems];
 #pragma unroll
         for (int j = 0; j < kDItems; ++j) {
-            if (i[j] < n && f[j] < n) v[j] = MODE == Mode::Gather ? __ldg(in + f[j]) : __ldg(in + i[j]);
+            if (i[j] < n && f[j] < n) v[j] = MODE == Mode::Gather ? __ldg(in + f[j]) : __ldcs(in + i[j]);
         }
 #pragma unroll
         for (int j = 0; j < kDItems; ++j) {

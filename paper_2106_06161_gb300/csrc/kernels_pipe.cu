@@ -1,10 +1,9 @@
-// Pipelined single pass of Algorithm 1 (pipe_kernel.cuh): the default shape
+// Pipelined single pass of Algorithm 1 (pipe_kernel.cuh): the default shapes
 // for every mode and width, the table of shapes the gather of 4-, 8- and
 // 16-byte elements can be tuned over, and the selection per width.
 //
-// Shape 0 is the default: eight compute warps of 8 items and three resident
-// CTAs per SM measured fastest on GB300 (more tiles in flight lengthen every
-// look-back walk; fewer warps hide less latency).  The other shapes are
+// Shape 0 is the default: eight compute warps of four indices a round, with
+// the rounds per tile set by the call (pipe_rounds).  The other shapes are
 // instantiated in kernels_pipe_tuned.cu and serve bshuffle_permute only.
 #include <atomic>
 #include <cstdint>
@@ -15,7 +14,7 @@
 namespace bsh {
 
 const PipeConfig kPipeConfigs[kNumPipeConfigs] = {
-    {8, 8, 3, 1}, {8, 4, 4, 1}, {8, 16, 2, 1}, {4, 8, 5, 1}, {16, 4, 2, 1}, {8, 8, 3, 0},
+    {8, 8, 4, 1}, {8, 4, 4, 1}, {8, 16, 3, 1}, {4, 8, 5, 1}, {16, 4, 2, 1}, {8, 8, 3, 0},
 };
 
 namespace {
@@ -32,10 +31,38 @@ int width_slot(uint32_t elem_bytes)
     }
 }
 
+// Rounds of four indices per thread in a tile of the default shape.  Four (3
+// CTAs per SM) where the kernel keeps the look-back warp busy: indices from
+// 2^21 on, and 4-byte gathers from there to 2^24, whose input the L2 holds.
+// Two (4 CTAs per SM) elsewhere: smaller domains have too few tiles to fill
+// the GPU with larger ones, larger gathers wait for memory, and the buffers
+// of wider elements would take the L1 that the gathers in flight need.
+// Measured on GB300, calls replayed from a graph, n = 15/16 of the domain,
+// four rounds against two: indices 2^20 14.0 / 12.7 us, 2^22 29.5 / 29.6,
+// 2^24 89.6 / 94.4; 4-byte gathers 2^20 15.2 / 14.8, 2^22 31.2 / 33.0, 2^24
+// 103 / 109, 2^25 328 / 316; 8-byte gathers 2^22 46.6 / 35.6, 2^24 422 / 186;
+// 8-byte scatters 2^22 39.4 / 39.2.
+int pipe_rounds(uint32_t elem_bytes, Mode mode, uint32_t k)
+{
+    const bool index = mode == Mode::Index32 || mode == Mode::Index64;
+    const bool gather4 = mode == Mode::Gather && elem_bytes == 4;
+    return (index && k >= 21) || (gather4 && k >= 21 && k <= 24) ? 4 : 2;
+}
+
 template <class T, Mode MODE>
 cudaError_t launch_default(const TileArgs &a, cudaStream_t stream)
 {
-    return pipe::launch_shape<T, MODE, 8, 8, 3, true>(a, stream);
+    constexpr bool index = MODE == Mode::Index32 || MODE == Mode::Index64;
+    if constexpr (index || (MODE == Mode::Gather && sizeof(T) == 4))
+        if (pipe_rounds(sizeof(T), MODE, a.g.k) == 4) return pipe::launch_shape<T, MODE, 8, 4, 4, 3, true>(a, stream);
+    // one round of eight for scatters, and for 8-byte gathers that the L2 does
+    // not hold: three CTAs of more accesses in flight each, instead of four
+    // (8-byte gathers at 2^24 - 5 208 / 203 us, scatters at 2^22 + 1 of 4
+    // bytes 76.4 / 74.6, 16-byte at 2^24 + 1 468 / 465)
+    if constexpr (MODE == Mode::Scatter || (MODE == Mode::Gather && sizeof(T) == 8))
+        if (MODE == Mode::Scatter || uint64_t{a.g.n} * sizeof(T) >= pipe::kTicketsAheadBytes)
+            return pipe::launch_shape<T, MODE, 8, 8, 1, 3, true>(a, stream);
+    return pipe::launch_shape<T, MODE, 8, 4, 2, 4, true>(a, stream);
 }
 
 }  // namespace
@@ -61,8 +88,9 @@ int selected_pipe_config(uint32_t elem_bytes)
     return slot < 0 ? 0 : g_pipe_selected[slot].load();
 }
 
-uint32_t pipe_tile_size(uint32_t, int config)
+uint32_t pipe_tile_size(uint32_t elem_bytes, int config, Mode mode, uint32_t k)
 {
+    if (config == 0) return 8u * 32u * 4u * static_cast<uint32_t>(pipe_rounds(elem_bytes, mode, k));
     const PipeConfig &c = kPipeConfigs[config >= 0 && config < kNumPipeConfigs ? config : 0];
     return static_cast<uint32_t>(c.warps * 32 * c.items);
 }

@@ -13,11 +13,11 @@ template <class T>
 cudaError_t launch_typed(const TileArgs &a, int config, cudaStream_t stream)
 {
     switch (config) {
-    case 1: return pipe::launch_shape<T, Mode::Gather, 8, 4, 4, true>(a, stream);
-    case 2: return pipe::launch_shape<T, Mode::Gather, 8, 16, 2, true>(a, stream);
-    case 3: return pipe::launch_shape<T, Mode::Gather, 4, 8, 5, true>(a, stream);
-    case 4: return pipe::launch_shape<T, Mode::Gather, 16, 4, 2, true>(a, stream);
-    case 5: return pipe::launch_shape<T, Mode::Gather, 8, 8, 3, false>(a, stream);
+    case 1: return pipe::launch_shape<T, Mode::Gather, 8, 4, 1, 4, true>(a, stream);
+    case 2: return pipe::launch_shape<T, Mode::Gather, 8, 4, 4, 3, true>(a, stream);
+    case 3: return pipe::launch_shape<T, Mode::Gather, 4, 4, 2, 5, true>(a, stream);
+    case 4: return pipe::launch_shape<T, Mode::Gather, 16, 4, 1, 2, true>(a, stream);
+    case 5: return pipe::launch_shape<T, Mode::Gather, 8, 4, 2, 3, false>(a, stream);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -80,14 +80,14 @@ cudaError_t launch_range_typed(const TileArgs &a, cudaStream_t stream)
 cudaError_t launch_permute_range(const TileArgs &a, uint32_t elem_bytes, cudaStream_t stream)
 {
     // tiles as counted by the caller: 2,048 domain indices (the plain
-    // kernel's 256 x 8 and the pipelined kernel's 8 warps x 32 x 8)
-    if (elem_tile_size(0) != 256u * 8u || pipe_tile_size(elem_bytes, 0) != 256u * 8u) return cudaErrorInvalidValue;
+    // kernel's 256 x 8 and the pipelined kernel's 8 warps x 32 x 4 x 2)
+    if (elem_tile_size(0) != 256u * 8u) return cudaErrorInvalidValue;
     switch (elem_bytes) {
     case 1: return launch_range_typed<uint8_t>(a, stream);
     case 2: return launch_range_typed<uint16_t>(a, stream);
-    case 4: return pipe::launch_shape<uint32_t, Mode::Gather, 8, 8, 3, true, true>(a, stream);
-    case 8: return pipe::launch_shape<unsigned long long, Mode::Gather, 8, 8, 3, true, true>(a, stream);
-    case 16: return pipe::launch_shape<uint4, Mode::Gather, 8, 8, 3, true, true>(a, stream);
+    case 4: return pipe::launch_shape<uint32_t, Mode::Gather, 8, 4, 2, 4, true, true>(a, stream);
+    case 8: return pipe::launch_shape<unsigned long long, Mode::Gather, 8, 4, 2, 4, true, true>(a, stream);
+    case 16: return pipe::launch_shape<uint4, Mode::Gather, 8, 4, 2, 4, true, true>(a, stream);
     default: return cudaErrorInvalidValue;
     }
 }

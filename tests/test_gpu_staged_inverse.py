@@ -58,7 +58,8 @@ def test_withheld_chunk_is_reported_and_the_next_call_exact(staged):
     assert np.array_equal(got, oracle.inverse(x, 3))
 
 
-@pytest.mark.parametrize("n,width", [(2**25 + 1, 8), (2**26 + 12345, 4), (2**24 + 1, 16), (2**28 + 12345, 8)])
+@pytest.mark.parametrize("n,width", [(2**24, 8), (2**25, 4), (2**24 - 5, 8), (2**25 + 1, 8), (2**26 + 12345, 4),
+                                     (2**24 - 12345, 16), (2**24 + 1, 16), (2**28 + 12345, 8)])
 def test_default_strategy_undoes_the_shuffle(bs, n, width):
     # at these sizes the default takes this path; the shuffle is checked
     # against the oracle elsewhere
