@@ -110,7 +110,6 @@ __device__ __forceinline__ void cipher_items_fixed(uint32_t (&left)[ITEMS], uint
 // What is left is bound by the ALU pipe (two LOP3 per even round, three per
 // odd one).  Measured on GB300, 2^28 evaluations, 8 items per thread: even k
 // 1.18 -> 0.80 ms, odd k 1.53 -> 1.27 ms.
-constexpr uint32_t kFloatMaxL = 10;
 constexpr uint32_t kFloatBase = 0x4B000000u;  // the pattern of 2^23
 constexpr float kTwo23 = 8388608.0f;
 constexpr uint32_t kM0Lo = static_cast<uint32_t>(kM0);
@@ -147,7 +146,6 @@ __device__ __forceinline__ void floor_fma_items(uint32_t (&d)[ITEMS], const uint
 // modulo 2^12 in its smallest form, -365.  No 64-bit product is left: four
 // issue cycles of the FMA-heavy pipe per even round instead of six.  Measured
 // on GB300, 2^28 evaluations: even k 1.18 -> 1.00 ms, odd k 1.53 -> 1.39 ms.
-constexpr uint32_t kMixedMaxL = 12;
 constexpr float kTwo22 = 4194304.0f;
 constexpr uint32_t kMixedHi = (kM0Hi & ((1u << kMixedMaxL) - 1u)) - 1u;
 constexpr float kMixedFrac = 1.0f + static_cast<float>(kM0Lo >> 9) / kTwo23;
@@ -202,14 +200,18 @@ __device__ __forceinline__ void cipher_items_float(uint32_t (&left)[ITEMS], uint
     }
 }
 
-template <bool ODD, int ITEMS>
+// FORM: the form that the default round count takes (cipher_form of the left
+// half's width), or Any to choose it here.  Kernels that are mostly cipher are
+// instantiated per form, so that one form's registers do not set the others'
+// occupancy (the staged inverse's pass 1 lost 1-2 % with all of them inside).
+template <bool ODD, int ITEMS, CipherForm FORM = CipherForm::Any>
 __device__ __forceinline__ void cipher_items(uint32_t (&left)[ITEMS], uint32_t (&right)[ITEMS],
                                              const uint32_t *keys, uint32_t rounds, const Geometry &g)
 {
     if (rounds == kUnrolledRounds) {
-        if (g.L <= kFloatMaxL)
+        if (FORM == CipherForm::Float || (FORM == CipherForm::Any && g.L <= kFloatMaxL))
             cipher_items_float<ODD, false, ITEMS, kUnrolledRounds>(left, right, keys, g);
-        else if (g.L <= kMixedMaxL)
+        else if (FORM == CipherForm::Mixed || (FORM == CipherForm::Any && g.L <= kMixedMaxL))
             cipher_items_float<ODD, true, ITEMS, kUnrolledRounds>(left, right, keys, g);
         else
             cipher_items_fixed<ODD, ITEMS, kUnrolledRounds>(left, right, keys, g);

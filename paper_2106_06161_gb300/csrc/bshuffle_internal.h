@@ -44,6 +44,18 @@ struct Geometry {
     uint32_t lift_mul; // 2^L: multiplying by it moves bit 0 to bit L
 };
 
+// How a kernel evaluates the cipher's default 24 rounds: single-precision
+// products for left halves of at most 10 bits, the mixed form for at most 12
+// (it holds for fewer bits too), integer products for any; or whichever of
+// them the domain calls for.
+enum class CipherForm : int { Float = 0, Mixed = 1, Wide = 2, Any = 3 };
+constexpr uint32_t kFloatMaxL = 10;
+constexpr uint32_t kMixedMaxL = 12;
+inline CipherForm cipher_form(const Geometry &g)
+{
+    return g.L <= kFloatMaxL ? CipherForm::Float : g.L <= kMixedMaxL ? CipherForm::Mixed : CipherForm::Wide;
+}
+
 // Everything one fused tile launch needs, passed by value (param space).
 struct TileArgs {
     const void *in;

@@ -52,8 +52,8 @@ __device__ __forceinline__ double block_sum(double v, double *s_red)
     return t;  // valid in thread 0
 }
 
-template <bool ODD>
-__global__ void __launch_bounds__(kMcBlock, 4) mc_kernel(const __grid_constant__ McArgs a)
+template <bool ODD, CipherForm FORM>
+__global__ void __launch_bounds__(kMcBlock, 5) mc_kernel(const __grid_constant__ McArgs a)
 {
     __shared__ uint32_t s_keys[kMcWarps][kMaxRounds];
     __shared__ double s_red[kMcWarps];
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kMcBlock, 4) mc_kernel(const __grid_constant__
                 left[j] = i >> g.R;
                 right[j] = i & g.rmask;
             }
-            dev::cipher_items<ODD, kMcItems>(left, right, keys, a.rounds, g);
+            dev::cipher_items<ODD, kMcItems, FORM>(left, right, keys, a.rounds, g);
             if (a.n1 - running >= kMcChunk) {
                 // every kept index of the chunk belongs to the first group,
                 // whatever its rank
@@ -134,7 +134,7 @@ cudaError_t launch_mc(const McArgs &a, cudaStream_t stream)
     int ctas_cached = per_sm[device].load(std::memory_order_acquire);
     if (ctas_cached == 0) {
         int blocks = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, mc_kernel<true>, kMcBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, mc_kernel<true, CipherForm::Float>, kMcBlock, 0);
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
@@ -143,10 +143,16 @@ cudaError_t launch_mc(const McArgs &a, cudaStream_t stream)
     }
     const uint32_t want = (a.count + kMcWarps - 1) / kMcWarps;  // one warp per instance
     const uint32_t grid = want < static_cast<uint32_t>(ctas_cached) ? want : ctas_cached;
-    if (a.g.k & 1u)
-        mc_kernel<true><<<grid, kMcBlock, 0, stream>>>(a);
-    else
-        mc_kernel<false><<<grid, kMcBlock, 0, stream>>>(a);
+    const bool odd = (a.g.k & 1u) != 0u;
+    auto kernel = odd ? mc_kernel<true, CipherForm::Float> : mc_kernel<false, CipherForm::Float>;
+    switch (cipher_form(a.g)) {
+    case CipherForm::Float: break;
+    case CipherForm::Mixed:
+        kernel = odd ? mc_kernel<true, CipherForm::Mixed> : mc_kernel<false, CipherForm::Mixed>;
+        break;
+    default: kernel = odd ? mc_kernel<true, CipherForm::Wide> : mc_kernel<false, CipherForm::Wide>;
+    }
+    kernel<<<grid, kMcBlock, 0, stream>>>(a);
     return cudaGetLastError();
 }
 

@@ -33,8 +33,8 @@ constexpr int kSvWarps = kSvBlock / 32;
 constexpr int kSvItems = 8;
 constexpr uint32_t kSvChunk = 32 * kSvItems;
 
-template <bool ODD>
-__global__ void __launch_bounds__(kSvBlock) shapley_voting_kernel(const __grid_constant__ ShapleyArgs a)
+template <bool ODD, CipherForm FORM>
+__global__ void __launch_bounds__(kSvBlock, 5) shapley_voting_kernel(const __grid_constant__ ShapleyArgs a)
 {
     __shared__ uint32_t s_keys[kSvWarps][kMaxRounds];
     const uint32_t lane = threadIdx.x & 31u;
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kSvBlock) shapley_voting_kernel(const __grid_c
                 left[j] = i >> g.R;
                 right[j] = i & g.rmask;
             }
-            dev::cipher_items<ODD, kSvItems>(left, right, keys, a.rounds, g);
+            dev::cipher_items<ODD, kSvItems, FORM>(left, right, keys, a.rounds, g);
             uint32_t player[kSvItems], wt[kSvItems];
             uint64_t mine = 0;  // this lane's weights of the chunk
 #pragma unroll
@@ -99,7 +99,7 @@ cudaError_t launch_shapley_voting(const ShapleyArgs &a, cudaStream_t stream)
     int ctas_cached = per_sm[device].load(std::memory_order_acquire);
     if (ctas_cached == 0) {
         int blocks = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, shapley_voting_kernel<true>, kSvBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, shapley_voting_kernel<true, CipherForm::Float>, kSvBlock, 0);
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
@@ -109,10 +109,16 @@ cudaError_t launch_shapley_voting(const ShapleyArgs &a, cudaStream_t stream)
     const uint64_t cap = static_cast<uint64_t>(ctas_cached);
     const uint64_t want = (a.samples + kSvWarps - 1) / kSvWarps;  // one warp per sample
     const unsigned grid = static_cast<unsigned>(want < cap ? want : cap);
-    if (a.g.k & 1u)
-        shapley_voting_kernel<true><<<grid, kSvBlock, 0, stream>>>(a);
-    else
-        shapley_voting_kernel<false><<<grid, kSvBlock, 0, stream>>>(a);
+    const bool odd = (a.g.k & 1u) != 0u;
+    auto kernel = odd ? shapley_voting_kernel<true, CipherForm::Float> : shapley_voting_kernel<false, CipherForm::Float>;
+    switch (cipher_form(a.g)) {
+    case CipherForm::Float: break;
+    case CipherForm::Mixed:
+        kernel = odd ? shapley_voting_kernel<true, CipherForm::Mixed> : shapley_voting_kernel<false, CipherForm::Mixed>;
+        break;
+    default: kernel = odd ? shapley_voting_kernel<true, CipherForm::Wide> : shapley_voting_kernel<false, CipherForm::Wide>;
+    }
+    kernel<<<grid, kSvBlock, 0, stream>>>(a);
     return cudaGetLastError();
 }
 

@@ -115,7 +115,7 @@ __device__ __forceinline__ void block_exclusive_scan(const uint32_t *cnt, uint32
 // bucket is a window of domain indices and the last chunk is ragged.  The
 // round keys sit in kernel parameter space, so the unrolled 24 rounds read
 // them as constant operands.
-template <class T, bool ODD, bool FORWARD, int ITEMS, bool PADDED>
+template <class T, bool ODD, bool FORWARD, int ITEMS, bool PADDED, CipherForm FORM = CipherForm::Wide>
 __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
 {
     constexpr int kP1Items = ITEMS;
@@ -151,7 +151,7 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
         right[j] = b & g.rmask;
     }
     if constexpr (FORWARD)
-        dev::cipher_items<ODD, kP1Items>(left, right, a.keys, a.rounds, g);
+        dev::cipher_items<ODD, kP1Items, FORM>(left, right, a.keys, a.rounds, g);
     else
         dev::cipher_inverse_items<ODD, kP1Items>(left, right, a.keys, a.rounds, g);
     uint32_t dst[kP1Items], slot[kP1Items];
@@ -196,10 +196,11 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     }
 }
 
-template <class T, bool ODD, bool FORWARD, int ITEMS>
+// FORM: the forward cipher's (Mixed or Wide; the inverse cipher has one).
+template <class T, bool ODD, bool FORWARD, int ITEMS, CipherForm FORM = CipherForm::Wide>
 __global__ void __launch_bounds__(kP1Block) staged_bucket_kernel(const __grid_constant__ StagedArgs a)
 {
-    bucket_pass<T, ODD, FORWARD, ITEMS, false>(a);
+    bucket_pass<T, ODD, FORWARD, ITEMS, false, FORM>(a);
 }
 
 // The ranked form's P1, in kernels of its own so that their register
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kP1Block, BSHUFFLE_RANKED_P1_MIN_CTAS)
 // pass is bound by the cipher over the whole domain (the odd-k forward round)
 // and waits on the look-back: publishing the count before the window counts
 // took 2^28 + 12345 uint64 from 8.93 to 8.65 ms (single pass 10.7).
-template <class T, bool ODD, int ITEMS>
+template <class T, bool ODD, int ITEMS, CipherForm FORM>
 __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const __grid_constant__ StagedArgs a)
 {
     constexpr uint32_t kTile = kP1Block * ITEMS;
@@ -277,7 +278,7 @@ __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const _
         left[j] = i >> g.R;
         right[j] = i & g.rmask;
     }
-    dev::cipher_items<ODD, ITEMS>(left, right, a.keys, a.rounds, g);
+    dev::cipher_items<ODD, ITEMS, FORM>(left, right, a.keys, a.rounds, g);
     uint32_t dst[ITEMS], mask[ITEMS], slot[ITEMS];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
@@ -630,6 +631,7 @@ cudaError_t launch_p1(const StagedArgs &a, int device, cudaStream_t stream)
 {
     using Kernel = void (*)(StagedArgs);
     Kernel odd, even;
+    int form = 0;
     if constexpr (PADDED && ITEMS == 16 && sizeof(T) <= 8) {
         odd = staged_rank_bucket16_kernel<T, true>;
         even = staged_rank_bucket16_kernel<T, false>;
@@ -639,14 +641,20 @@ cudaError_t launch_p1(const StagedArgs &a, int device, cudaStream_t stream)
     } else {
         odd = staged_bucket_kernel<T, true, FORWARD, ITEMS>;
         even = staged_bucket_kernel<T, false, FORWARD, ITEMS>;
+        if constexpr (FORWARD && ITEMS == 8)  // 16 items: over 2^26 elements
+            if (cipher_form(a.g) != CipherForm::Wide) {
+                odd = staged_bucket_kernel<T, true, FORWARD, ITEMS, CipherForm::Mixed>;
+                even = staged_bucket_kernel<T, false, FORWARD, ITEMS, CipherForm::Mixed>;
+                form = 1;
+            }
     }
-    static std::atomic<bool> configured[64];  // attribute set on this device
-    if (!configured[device].load(std::memory_order_acquire)) {
+    static std::atomic<bool> configured[2][64];  // attribute set on this device
+    if (!configured[form][device].load(std::memory_order_acquire)) {
         const int most = static_cast<int>(p1_smem_bytes<T, ITEMS>(4096));
         cudaError_t e = cudaFuncSetAttribute(odd, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(even, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
-        configured[device].store(true, std::memory_order_release);
+        configured[form][device].store(true, std::memory_order_release);
     }
     const size_t dyn = p1_smem_bytes<T, ITEMS>(a.num_dst);
     const uint64_t tile = uint64_t{kP1Block} * ITEMS;
@@ -700,10 +708,11 @@ cudaError_t launch_rank(const StagedArgs &a, int device, cudaStream_t stream)
 
 
 // P1 of the inverse shuffle for n < 2^k.
-template <class T, int ITEMS>
+template <class T, int ITEMS, CipherForm FORM>
 cudaError_t launch_inverse_p1(const StagedArgs &a, int device, cudaStream_t stream)
 {
-    const auto odd = staged_inverse_bucket_kernel<T, true, ITEMS>, even = staged_inverse_bucket_kernel<T, false, ITEMS>;
+    const auto odd = staged_inverse_bucket_kernel<T, true, ITEMS, FORM>;
+    const auto even = staged_inverse_bucket_kernel<T, false, ITEMS, FORM>;
     static std::atomic<bool> configured[64];  // attribute set on this device
     if (!configured[device].load(std::memory_order_acquire)) {
         const int most = static_cast<int>(p1_smem_bytes<T, ITEMS>(4096));
@@ -740,10 +749,14 @@ cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t strea
         if constexpr (!FORWARD)
             e = items == 16 ? launch_p1<T, false, 16, true>(a, device, stream)
                             : launch_p1<T, false, 8, true>(a, device, stream);
+        else if (cipher_form(a.g) != CipherForm::Wide)
+            e = items == 16 ? cudaErrorInvalidValue  // over 2 GiB, so over 2^26 elements
+                            : launch_inverse_p1<T, 8, CipherForm::Mixed>(a, device, stream);
         else if constexpr (sizeof(T) <= 8)
-            e = items == 16 ? launch_inverse_p1<T, 16>(a, device, stream) : launch_inverse_p1<T, 8>(a, device, stream);
+            e = items == 16 ? launch_inverse_p1<T, 16, CipherForm::Wide>(a, device, stream)
+                            : launch_inverse_p1<T, 8, CipherForm::Wide>(a, device, stream);
         else
-            e = launch_inverse_p1<T, 8>(a, device, stream);
+            e = launch_inverse_p1<T, 8, CipherForm::Wide>(a, device, stream);
     } else if constexpr (sizeof(T) <= 8) {
         e = items == 16 ? launch_p1<T, FORWARD, 16, false>(a, device, stream)
                         : launch_p1<T, FORWARD, 8, false>(a, device, stream);

@@ -217,7 +217,8 @@ __global__ void __launch_bounds__(kKBlock) sample_ranks_kernel(const __grid_cons
                 left[j] = i >> g.R;
                 right[j] = i & g.rmask;
             }
-            dev::cipher_items<ODD, kRItems>(left, right, keys, a.rounds, g);
+            dev::cipher_items<ODD, kRItems, CipherForm::Float>(  // n <= 4096
+                left, right, keys, a.rounds, g);
 #pragma unroll
             for (int j = 0; j < kRItems; ++j) {
                 const uint32_t i = base + static_cast<uint32_t>(j * 32) + lane;
