@@ -282,13 +282,79 @@ __device__ __forceinline__ void cipher_inverse_items_fixed(uint32_t (&left)[ITEM
     for (int j = 0; j < ITEMS; ++j) right[j] &= g.rmask;
 }
 
-template <bool ODD, int ITEMS>
+// Even k, default rounds: the high product word without its 32 x 32 -> 64-bit
+// product (four of the round's eight issue cycles on the FMA-heavy pipe).  As
+// in cipher_items_float the left half is kept as X = 2^23 + left, and the high
+// word's low L bits are left * (M0hi - 1) + floor(left * 1.694...), now for
+// every L up to 16: the multiplier (2^32 + M0lo) / 2^32 is split into 217 / 128
+// (2^23 of it is a multiple of 2^16, so that the pattern adds nothing below bit
+// L) and a negative rest of 22 bits, so both FMAs, rounded down, give the exact
+// floor (the first one's value is rounded to a grid that holds the multiples of
+// 2^-7 at which the second one's floor steps).  The forward round gains nothing
+// from this (its product gives the low word too).  MIXED: at most 12 bits, one
+// FMA.  Measured on GB300, 2^28 evaluations at k = 28: 1.35 -> 1.15 ms.
+constexpr float kFracTop = 217.0f / 128.0f;
+constexpr float kFracRest = -(static_cast<float>(0xB2000000u - kM0Lo) / 4294967296.0f);
+static_assert(0xB2000000u - kM0Lo < (1u << 22), "the rest of the multiplier is exact in a float");
+
+// d[j] = floor(x[j] * mul + d[j]) for floats kept as patterns.
+template <int ITEMS>
+__device__ __forceinline__ void floor_fma_onto_items(uint32_t (&d)[ITEMS], const uint32_t (&x)[ITEMS], float mul)
+{
+    static_assert(ITEMS % 2 == 0, "two items an instruction");
+    const uint32_t m = __float_as_uint(mul);
+#pragma unroll
+    for (int j = 0; j < ITEMS; j += 2)
+        asm("{\n\t.reg .b64 x, m, c;\n\t"
+            "mov.b64 x, {%2, %3};\n\tmov.b64 m, {%4, %4};\n\tmov.b64 c, {%0, %1};\n\t"
+            "fma.rm.f32x2 x, x, m, c;\n\t"
+            "mov.b64 {%0, %1}, x;\n\t}"
+            : "+r"(d[j]), "+r"(d[j + 1])
+            : "r"(x[j]), "r"(x[j + 1]), "r"(m));
+}
+
+template <bool MIXED, int ITEMS, int ROUNDS>
+__device__ __forceinline__ void cipher_inverse_items_float(uint32_t (&left)[ITEMS], uint32_t (&right)[ITEMS],
+                                                           const uint32_t *keys, const Geometry &g)
+{
+    const uint32_t lmask = g.lmask;
+    const float frac_add = MIXED ? -__uint2float_rn(kMixedFracInt & lmask) : 0.0f;
+#pragma unroll
+    for (int r = ROUNDS - 1; r >= 0; --r) {
+        const uint32_t key = keys[r];
+        uint32_t old_left[ITEMS], hi[ITEMS];
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) old_left[j] = ((right[j] * kM0InvLo) & lmask) | kFloatBase;
+        if constexpr (MIXED) {
+            floor_fma_items(hi, old_left, kMixedFrac, frac_add);
+        } else {
+            floor_fma_items(hi, old_left, kFracRest, -kTwo23 * kFracRest);
+            floor_fma_onto_items(hi, old_left, kFracTop);
+        }
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+            right[j] = left[j] ^ (old_left[j] * (kM0Hi - 1u) + hi[j]) ^ key;  // don't-care above bit L
+            left[j] = old_left[j];
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        left[j] &= lmask;
+        right[j] &= g.rmask;
+    }
+}
+
+// FORM as for cipher_items: Wide, or Mixed for left halves of at most 12 bits.
+template <bool ODD, int ITEMS, CipherForm FORM = CipherForm::Wide>
 __device__ __forceinline__ void cipher_inverse_items(uint32_t (&left)[ITEMS], uint32_t (&right)[ITEMS],
                                                      const uint32_t *keys, uint32_t rounds, const Geometry &g)
 {
-    if (rounds == kUnrolledRounds)
-        cipher_inverse_items_fixed<ODD, ITEMS, kUnrolledRounds>(left, right, keys, g);
-    else
+    if (rounds == kUnrolledRounds) {
+        if constexpr (ODD)
+            cipher_inverse_items_fixed<ODD, ITEMS, kUnrolledRounds>(left, right, keys, g);
+        else
+            cipher_inverse_items_float<FORM == CipherForm::Mixed, ITEMS, kUnrolledRounds>(left, right, keys, g);
+    } else
         cipher_inverse_items_loop<ODD, ITEMS>(left, right, keys, rounds, g);
 }
 

@@ -153,7 +153,7 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     if constexpr (FORWARD)
         dev::cipher_items<ODD, kP1Items, FORM>(left, right, a.keys, a.rounds, g);
     else
-        dev::cipher_inverse_items<ODD, kP1Items>(left, right, a.keys, a.rounds, g);
+        dev::cipher_inverse_items<ODD, kP1Items, FORM>(left, right, a.keys, a.rounds, g);
     uint32_t dst[kP1Items], slot[kP1Items];
 #pragma unroll
     for (int j = 0; j < kP1Items; ++j) dst[j] = (left[j] << g.R) | right[j];  // f^-1(b) (or f(b)): its slot
@@ -196,7 +196,7 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     }
 }
 
-// FORM: the forward cipher's (Mixed or Wide; the inverse cipher has one).
+// FORM: Mixed or Wide (the inverse cipher's odd-k round has one form).
 template <class T, bool ODD, bool FORWARD, int ITEMS, CipherForm FORM = CipherForm::Wide>
 __global__ void __launch_bounds__(kP1Block) staged_bucket_kernel(const __grid_constant__ StagedArgs a)
 {
@@ -641,9 +641,9 @@ cudaError_t launch_p1(const StagedArgs &a, int device, cudaStream_t stream)
     } else {
         odd = staged_bucket_kernel<T, true, FORWARD, ITEMS>;
         even = staged_bucket_kernel<T, false, FORWARD, ITEMS>;
-        if constexpr (FORWARD && ITEMS == 8)  // 16 items: over 2^26 elements
+        if constexpr (ITEMS == 8)  // 16 items: over 2^26 elements
             if (cipher_form(a.g) != CipherForm::Wide) {
-                odd = staged_bucket_kernel<T, true, FORWARD, ITEMS, CipherForm::Mixed>;
+                if constexpr (FORWARD) odd = staged_bucket_kernel<T, true, FORWARD, ITEMS, CipherForm::Mixed>;
                 even = staged_bucket_kernel<T, false, FORWARD, ITEMS, CipherForm::Mixed>;
                 form = 1;
             }

@@ -66,6 +66,39 @@ def test_mixed_products_exact(L):
     assert np.array_equal(odd & 1, [(w >> (L - 1)) & 1 for w in wide])
 
 
+@pytest.mark.parametrize("L", range(2, 17))
+def test_split_high_word_exact(L):
+    # the inverse round's high word: 1.694... as 217/128 and a negative rest,
+    # both multiply-adds rounded down, the first one to 24 significant bits
+    left = np.arange(1 << L, dtype=np.int64)
+    mask = (1 << L) - 1
+    rest = LO - 0xB2000000
+    assert -(1 << 22) < rest < 0 and float(np.float32(rest)) == rest
+    exact = -left * rest                                   # in units of 2^-32, non-negative
+    drop = np.maximum(np.array([int(v).bit_length() for v in exact]) - 24, 0)
+    y = -(((exact + (1 << drop) - 1) >> drop) << drop)      # towards minus infinity
+    frac = _pattern((left + TWO23) * 217 * (1 << 25) + y, 32)
+    hi = frac + left * (HI - 1)
+    assert np.array_equal(hi & mask, [((int(v) * M0) >> 32) & mask for v in left])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("k", range(13, 27))
+def test_staged_shuffle_uses_the_inverse_cipher(k):
+    import torch
+
+    import paper_2106_06161_gb300 as bs
+    bs.bshuffle_set_strategy(bs.BSHUFFLE_STRATEGY_STAGED)
+    try:
+        for width, dtype in ((4, torch.int32), (8, torch.int64)):
+            x = torch.arange(1 << k, dtype=dtype, device="cuda")
+            got = bs.permute(x, 77)
+            assert bs.get_error() == 0
+            assert torch.equal(got, bs.indices(1 << k, 77, dtype=dtype))   # the forward cipher
+    finally:
+        bs.bshuffle_set_strategy(bs.BSHUFFLE_STRATEGY_AUTO)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("k", range(4, 27))
 def test_indices_match_oracle(k):
