@@ -365,11 +365,11 @@ int bshuffle_release_workspaces(void);
  *       (a look-back gives each chunk's first source slot) and buckets by
  *       output window; workspace n * (4 + elem_bytes) bytes plus a little.
  *   BSHUFFLE_STRATEGY_PIPELINED  the single pass with its look-back taken
- *       off the compute warps, for gathers and scatters of 4, 8 and 16-byte
- *       elements and for indices (other calls run the plain single pass):
+ *       off the compute warps, for gathers and scatters of 1, 2, 4, 8 and
+ *       16-byte elements and for indices (rows run the plain single pass):
  *       persistent CTAs; eight compute warps evaluate the bijection of a tile
- *       and copy its kept elements into shared memory with cp.async, then
- *       store the previous tile, which a ninth warp has meanwhile ranked
+ *       and copy its kept elements into shared memory with cp.async (1- and
+ *       2-byte elements are read when they are stored), then store the previous tile, which a ninth warp has meanwhile ranked
  *       with the look-back.  Same memory traffic and workspace as the single
  *       pass.
  *   BSHUFFLE_STRATEGY_AUTO (default)  staged when it applies and

@@ -33,7 +33,8 @@ int width_slot(uint32_t elem_bytes)
 
 // Rounds of four indices per thread in a tile of the default shape.  Four (3
 // CTAs per SM) where the kernel keeps the look-back warp busy: indices from
-// 2^21 on, and 4-byte gathers from there to 2^24, whose input the L2 holds.
+// 2^21 on, 4-byte gathers from there to 2^24, whose input the L2 holds, and
+// narrower ones from 2^25 on.
 // Two (4 CTAs per SM) elsewhere: smaller domains have too few tiles to fill
 // the GPU with larger ones, larger gathers wait for memory, and the buffers
 // of wider elements would take the L1 that the gathers in flight need.
@@ -41,19 +42,23 @@ int width_slot(uint32_t elem_bytes)
 // four rounds against two: indices 2^20 14.0 / 12.7 us, 2^22 29.5 / 29.6,
 // 2^24 89.6 / 94.4; 4-byte gathers 2^20 15.2 / 14.8, 2^22 31.2 / 33.0, 2^24
 // 103 / 109, 2^25 328 / 316; 8-byte gathers 2^22 46.6 / 35.6, 2^24 422 / 186;
-// 8-byte scatters 2^22 39.4 / 39.2.
+// 8-byte scatters 2^22 39.4 / 39.2.  Two-byte gathers, four / two: 2^22 + 1
+// 81.0 / 78.0, 2^24 + 1 263 / 269, 2^26 + 1 1087 / 1134, 2^28 + 1 4951 / 4955
+// (in the plain fused kernel 84, 286, 1250 and 7099; two-byte scatters at 2^22
+// + 1 81 against 88 there, at 2^26 + 1 1206 against 1454).
 int pipe_rounds(uint32_t elem_bytes, Mode mode, uint32_t k)
 {
     const bool index = mode == Mode::Index32 || mode == Mode::Index64;
     const bool gather4 = mode == Mode::Gather && elem_bytes == 4;
-    return (index && k >= 21) || (gather4 && k >= 21 && k <= 24) ? 4 : 2;
+    const bool narrow = mode == Mode::Gather && elem_bytes < 4;
+    return (index && k >= 21) || (gather4 && k >= 21 && k <= 24) || (narrow && k >= 25) ? 4 : 2;
 }
 
 template <class T, Mode MODE>
 cudaError_t launch_default(const TileArgs &a, cudaStream_t stream)
 {
     constexpr bool index = MODE == Mode::Index32 || MODE == Mode::Index64;
-    if constexpr (index || (MODE == Mode::Gather && sizeof(T) == 4))
+    if constexpr (index || (MODE == Mode::Gather && sizeof(T) <= 4))
         if (pipe_rounds(sizeof(T), MODE, a.g.k) == 4) return pipe::launch_shape<T, MODE, 8, 4, 4, 3, true>(a, stream);
     // one round of eight for scatters, and for 8-byte gathers that the L2 does
     // not hold: three CTAs of more accesses in flight each, instead of four
@@ -99,7 +104,8 @@ bool pipe_supports(Mode mode, uint32_t elem_bytes)
 {
     switch (mode) {
     case Mode::Gather:
-    case Mode::Scatter: return elem_bytes == 4 || elem_bytes == 8 || elem_bytes == 16;
+    case Mode::Scatter:
+        return elem_bytes == 1 || elem_bytes == 2 || elem_bytes == 4 || elem_bytes == 8 || elem_bytes == 16;
     case Mode::Index32:
     case Mode::Index64: return true;
     }
@@ -117,6 +123,8 @@ cudaError_t launch_pipe(const TileArgs &a, Mode mode, uint32_t elem_bytes, int c
     case Mode::Index64: return launch_default<unsigned long long, Mode::Index64>(a, stream);
     case Mode::Gather:
         switch (elem_bytes) {
+        case 1: return launch_default<unsigned char, Mode::Gather>(a, stream);
+        case 2: return launch_default<unsigned short, Mode::Gather>(a, stream);
         case 4: return launch_default<unsigned int, Mode::Gather>(a, stream);
         case 8: return launch_default<unsigned long long, Mode::Gather>(a, stream);
         case 16: return launch_default<uint4, Mode::Gather>(a, stream);
@@ -124,6 +132,8 @@ cudaError_t launch_pipe(const TileArgs &a, Mode mode, uint32_t elem_bytes, int c
         }
     case Mode::Scatter:
         switch (elem_bytes) {
+        case 1: return launch_default<unsigned char, Mode::Scatter>(a, stream);
+        case 2: return launch_default<unsigned short, Mode::Scatter>(a, stream);
         case 4: return launch_default<unsigned int, Mode::Scatter>(a, stream);
         case 8: return launch_default<unsigned long long, Mode::Scatter>(a, stream);
         case 16: return launch_default<uint4, Mode::Scatter>(a, stream);

@@ -1,5 +1,5 @@
-// Pipelined single pass of Algorithm 1 (gather and scatter of 4-, 8- and
-// 16-byte elements, and the index output): the same output as the fused tile
+// Pipelined single pass of Algorithm 1 (gather and scatter of 1- to 16-byte
+// elements, and the index output): the same output as the fused tile
 // kernel, with the inter-tile look-back taken off the compute warps' path.
 //
 // In the plain fused kernel every warp of a tile waits while one warp looks
@@ -81,11 +81,19 @@ struct PipeShared {
 // 90 us ahead, 107 in the form with a barrier).
 constexpr uint64_t kTicketsAheadBytes = uint64_t{96} << 20;
 
-// What a tile buffer holds per kept index: the gathered element (gather), or
-// the image itself, which the store writes (indices) or takes as the target
-// of the element that it reads then (scatter: out[f(i_j)] = in[j]).
+// Whether the gathers run with cp.async while the tile waits for its rank: it
+// copies 4, 8 or 16 bytes.  Narrower elements are read when they are stored.
+// (Copying the aligned word around each, with its bit offset in a byte beside
+// it, was no faster: 2-byte gathers at 2^26 + 1 1126 / 1134 us, at 2^27 - 5
+// 1909 / 1770.)
 template <class T, Mode MODE>
-using PipeSlot = typename std::conditional<MODE == Mode::Gather, T, uint32_t>::type;
+constexpr bool kAsyncGather = MODE == Mode::Gather && sizeof(T) >= 4;
+
+// What a tile buffer holds per kept index: the gathered element, or the image
+// itself, which the store writes (indices), reads from (1- and 2-byte gathers)
+// or writes the element that it reads then to (scatter: out[f(i_j)] = in[j]).
+template <class T, Mode MODE>
+using PipeSlot = typename std::conditional<kAsyncGather<T, MODE>, T, uint32_t>::type;
 
 // MINB: resident CTAs per SM the register budget targets; UNROLL: the
 // default round count runs fully unrolled (else every count runs in a loop).
@@ -96,7 +104,7 @@ template <class T, Mode MODE, bool ODD, int NW, int ITEMS, int SUB, int MINB, bo
 __global__ void __launch_bounds__((NW + 1) * 32, MINB) pipe_tile_kernel(const __grid_constant__ TileArgs a)
 {
     using S = PipeSlot<T, MODE>;
-    constexpr bool ASYNC = MODE == Mode::Gather;
+    constexpr bool ASYNC = kAsyncGather<T, MODE>;
     constexpr uint32_t kWarpTile = 32 * ITEMS;  // domain indices of one compute warp and round
     constexpr uint32_t TILE = NW * SUB * kWarpTile;
     static_assert(NW * SUB <= 32, "one lane of the look-back warp per count");
@@ -165,7 +173,19 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) pipe_tile_kernel(const __
                     if (lane == 0) dev::record_error(a.ws, dev::kErrDeviceBounds, uint64_t{dst} + count - 1u);
                     count = dst < limit ? limit - dst : 0u;
                 }
-                if constexpr (MODE == Mode::Scatter) {
+                if constexpr (MODE == Mode::Gather && !ASYNC) {
+                    T v[ITEMS];
+#pragma unroll
+                    for (int j = 0; j < ITEMS; ++j) {
+                        const uint32_t e = static_cast<uint32_t>(j * 32) + lane;
+                        if (e < count) v[j] = __ldg(in + buf[e]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < ITEMS; ++j) {
+                        const uint32_t e = static_cast<uint32_t>(j * 32) + lane;
+                        if (e < count) out[uint64_t{dst} + e] = v[j];
+                    }
+                } else if constexpr (MODE == Mode::Scatter) {
                     // coalesced reads of this tile's slots, then the random writes
                     T v[ITEMS];
 #pragma unroll
