@@ -48,12 +48,19 @@ struct Geometry {
 // products for left halves of at most 10 bits, the mixed form for at most 12
 // (it holds for fewer bits too), integer products for any; or whichever of
 // them the domain calls for.
-enum class CipherForm : int { Float = 0, Mixed = 1, Wide = 2, Any = 3 };
+// Short: Float for runs of indices that do not share their left half
+// (dev::cipher_run).
+enum class CipherForm : int { Float = 0, Mixed = 1, Wide = 2, Any = 3, Short = 4 };
 constexpr uint32_t kFloatMaxL = 10;
 constexpr uint32_t kMixedMaxL = 12;
 inline CipherForm cipher_form(const Geometry &g)
 {
     return g.L <= kFloatMaxL ? CipherForm::Float : g.L <= kMixedMaxL ? CipherForm::Mixed : CipherForm::Wide;
+}
+// The form for runs whose groups span `span` indices, a power of two.
+inline CipherForm cipher_run_form(const Geometry &g, uint32_t span)
+{
+    return g.lmask < span - 1u ? CipherForm::Short : cipher_form(g);
 }
 
 // Everything one fused tile launch needs, passed by value (param space).

@@ -52,7 +52,10 @@ __global__ void __launch_bounds__(kDBlock) direct_elem_kernel(const __grid_const
     uint32_t i[kDItems], f[kDItems];
 #pragma unroll
     for (int j = 0; j < kDItems; ++j) i[j] = base + static_cast<uint32_t>(j * kDBlock);
-    images<ODD, kDItems>(a, i, f);
+    uint32_t left[kDItems], right[kDItems];
+    dev::cipher_run_wide<ODD, kDItems, kDBlock, CipherForm::Any>(left, right, base, a.keys, a.rounds, a.g);
+#pragma unroll
+    for (int j = 0; j < kDItems; ++j) f[j] = (left[j] << a.g.R) | right[j];
 
     if constexpr (MODE == Mode::Index32 || MODE == Mode::Index64) {
         using I = typename std::conditional<MODE == Mode::Index32, uint32_t, unsigned long long>::type;

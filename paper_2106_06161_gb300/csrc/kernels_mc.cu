@@ -16,7 +16,8 @@
 // missing from the first group, a chunk's kept elements all belong to it, and
 // one warp reduction counts them.  The kernel is bound by the ALU pipe (the
 // cipher's rounds; 73 % busy) beside the FP64 pipe (one conversion and one
-// addition per index; 68 %).  10,000 x 100,000 on GB300: 4.16 -> 3.81 ms.
+// addition per index; 68 %).  10,000 x 100,000 on GB300: 4.16 -> 3.81 ms with
+// the ranks left out, 3.87 -> 3.71 with the first round shared (cipher_run).
 // Handing the instances to the warps by ticket, or running fewer warps in
 // whole rounds, gained nothing (3.84 and 4.11 ms).
 #include <atomic>
@@ -81,13 +82,8 @@ __global__ void __launch_bounds__(kMcBlock, 5) mc_kernel(const __grid_constant__
         double s1 = 0.0;
         for (uint64_t base = 0; base < g.domain && running < a.n1; base += kMcChunk) {
             uint32_t left[kMcItems], right[kMcItems];
-#pragma unroll
-            for (int j = 0; j < kMcItems; ++j) {
-                const uint32_t i = static_cast<uint32_t>(base) + static_cast<uint32_t>(j * 32) + lane;
-                left[j] = i >> g.R;
-                right[j] = i & g.rmask;
-            }
-            dev::cipher_items<ODD, kMcItems, FORM>(left, right, keys, a.rounds, g);
+            dev::cipher_run<ODD, kMcItems, 32, kMcItems, FORM>(left, right, static_cast<uint32_t>(base) + lane, keys,
+                                                        a.rounds, g);
             if (a.n1 - running >= kMcChunk) {
                 // every kept index of the chunk belongs to the first group,
                 // whatever its rank
@@ -145,8 +141,11 @@ cudaError_t launch_mc(const McArgs &a, cudaStream_t stream)
     const uint32_t grid = want < static_cast<uint32_t>(ctas_cached) ? want : ctas_cached;
     const bool odd = (a.g.k & 1u) != 0u;
     auto kernel = odd ? mc_kernel<true, CipherForm::Float> : mc_kernel<false, CipherForm::Float>;
-    switch (cipher_form(a.g)) {
+    switch (cipher_run_form(a.g, kMcItems * 32)) {
     case CipherForm::Float: break;
+    case CipherForm::Short:
+        kernel = odd ? mc_kernel<true, CipherForm::Short> : mc_kernel<false, CipherForm::Short>;
+        break;
     case CipherForm::Mixed:
         kernel = odd ? mc_kernel<true, CipherForm::Mixed> : mc_kernel<false, CipherForm::Mixed>;
         break;

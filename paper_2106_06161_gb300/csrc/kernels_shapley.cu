@@ -16,7 +16,8 @@
 // earlier one adds its weight by two warp reductions, where an ordered 64-bit
 // scan of each 32 players (ten shuffles) took a quarter of the time.  The
 // kernel is bound by the ALU pipe (81 % busy, the cipher's rounds).  10,000
-// players, 100,000 orders on GB300: 4.63 -> 3.09 ms.
+// players, 100,000 orders on GB300: 4.63 -> 3.04 ms, and 3.04 -> 2.93 with the
+// first round shared (cipher_run).
 #include <atomic>
 #include <cstdint>
 
@@ -31,6 +32,7 @@ using dev::kFull;
 constexpr int kSvBlock = 256;
 constexpr int kSvWarps = kSvBlock / 32;
 constexpr int kSvItems = 8;
+constexpr int kSvGroup = 4;  // indices that share the cipher's first round (from 2^14 players on)
 constexpr uint32_t kSvChunk = 32 * kSvItems;
 
 template <bool ODD, CipherForm FORM>
@@ -50,13 +52,8 @@ __global__ void __launch_bounds__(kSvBlock, 5) shapley_voting_kernel(const __gri
         uint64_t carry = 0;  // weight of every kept player of the earlier chunks
         for (uint64_t base = 0; base < g.domain && carry < a.quota; base += kSvChunk) {
             uint32_t left[kSvItems], right[kSvItems];
-#pragma unroll
-            for (int j = 0; j < kSvItems; ++j) {
-                const uint32_t i = static_cast<uint32_t>(base) + static_cast<uint32_t>(j * 32) + lane;
-                left[j] = i >> g.R;
-                right[j] = i & g.rmask;
-            }
-            dev::cipher_items<ODD, kSvItems, FORM>(left, right, keys, a.rounds, g);
+            dev::cipher_run<ODD, kSvItems, 32, kSvGroup, FORM>(left, right, static_cast<uint32_t>(base) + lane, keys,
+                                                        a.rounds, g);
             uint32_t player[kSvItems], wt[kSvItems];
             uint64_t mine = 0;  // this lane's weights of the chunk
 #pragma unroll
@@ -111,8 +108,11 @@ cudaError_t launch_shapley_voting(const ShapleyArgs &a, cudaStream_t stream)
     const unsigned grid = static_cast<unsigned>(want < cap ? want : cap);
     const bool odd = (a.g.k & 1u) != 0u;
     auto kernel = odd ? shapley_voting_kernel<true, CipherForm::Float> : shapley_voting_kernel<false, CipherForm::Float>;
-    switch (cipher_form(a.g)) {
+    switch (cipher_run_form(a.g, kSvGroup * 32)) {
     case CipherForm::Float: break;
+    case CipherForm::Short:
+        kernel = odd ? shapley_voting_kernel<true, CipherForm::Short> : shapley_voting_kernel<false, CipherForm::Short>;
+        break;
     case CipherForm::Mixed:
         kernel = odd ? shapley_voting_kernel<true, CipherForm::Mixed> : shapley_voting_kernel<false, CipherForm::Mixed>;
         break;

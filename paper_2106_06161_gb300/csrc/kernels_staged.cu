@@ -147,11 +147,11 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     for (int j = 0; j < kP1Items; ++j) {
         const uint32_t b = first + static_cast<uint32_t>(j * kP1Block) + tid;
         if (!PADDED || b < g.n) val[j] = __ldcs(in + b);
-        left[j] = b >> g.R;  // beyond a padded n: never used
-        right[j] = b & g.rmask;
+        if (!FORWARD) left[j] = b >> g.R;  // beyond a padded n: never used
+        if (!FORWARD) right[j] = b & g.rmask;
     }
     if constexpr (FORWARD)
-        dev::cipher_items<ODD, kP1Items, FORM>(left, right, a.keys, a.rounds, g);
+        dev::cipher_run_wide<ODD, kP1Items, kP1Block, FORM>(left, right, first + tid, a.keys, a.rounds, g);
     else
         dev::cipher_inverse_items<ODD, kP1Items, FORM>(left, right, a.keys, a.rounds, g);
     uint32_t dst[kP1Items], slot[kP1Items];
@@ -272,13 +272,7 @@ __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const _
     // the domain is a multiple of the chunk
     const uint32_t base = tile * kTile + tid;
     uint32_t left[ITEMS], right[ITEMS];
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t i = base + static_cast<uint32_t>(j * kP1Block);
-        left[j] = i >> g.R;
-        right[j] = i & g.rmask;
-    }
-    dev::cipher_items<ODD, ITEMS, FORM>(left, right, a.keys, a.rounds, g);
+    dev::cipher_run_wide<ODD, ITEMS, kP1Block, FORM>(left, right, base, a.keys, a.rounds, g);
     uint32_t dst[ITEMS], mask[ITEMS], slot[ITEMS];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {

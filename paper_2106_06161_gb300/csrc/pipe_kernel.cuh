@@ -234,16 +234,15 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) pipe_tile_kernel(const __
                     // indices of the part inside the domain
                     const uint32_t live = end - start < kWarpTile ? static_cast<uint32_t>(end - start) : kWarpTile;
                     uint32_t left[ITEMS], right[ITEMS];
-#pragma unroll
-                    for (int j = 0; j < ITEMS; ++j) {
-                        const uint32_t i = base + static_cast<uint32_t>(j * 32);
-                        left[j] = i >> a.g.R;
-                        right[j] = i & a.g.rmask;
+                    if constexpr (UNROLL && !RANGE) {  // a range may start anywhere
+                        dev::cipher_run<ODD, ITEMS, 32>(left, right, base, a.keys, a.rounds, a.g);
+                    } else {
+                        dev::split_items<ITEMS, 32>(left, right, base, a.g);
+                        if constexpr (UNROLL)
+                            dev::cipher_items<ODD, ITEMS>(left, right, a.keys, a.rounds, a.g);
+                        else
+                            dev::cipher_items_loop<ODD, ITEMS>(left, right, a.keys, a.rounds, a.g);
                     }
-                    if constexpr (UNROLL)
-                        dev::cipher_items<ODD, ITEMS>(left, right, a.keys, a.rounds, a.g);
-                    else
-                        dev::cipher_items_loop<ODD, ITEMS>(left, right, a.keys, a.rounds, a.g);
                     S *buf = vals + static_cast<size_t>(b) * TILE + part * kWarpTile;
 #pragma unroll
                     for (int j = 0; j < ITEMS; ++j) {
