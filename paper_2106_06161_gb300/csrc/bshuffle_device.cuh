@@ -380,8 +380,9 @@ __device__ __forceinline__ void cipher_inverse_items_fixed(uint32_t (&left)[ITEM
     for (int j = 0; j < ITEMS; ++j) right[j] &= g.rmask;
 }
 
-// Even k, default rounds: the high product word without its 32 x 32 -> 64-bit
-// product (four of the round's eight issue cycles on the FMA-heavy pipe).  As
+// Default rounds: the high product word without its 32 x 32 -> 64-bit
+// product (four of the even round's eight issue cycles on the FMA-heavy pipe,
+// of the odd one's ten).  As
 // in cipher_items_float the left half is kept as X = 2^23 + left, and the high
 // word's low L bits are left * (M0hi - 1) + floor(left * 1.694...), now for
 // every L up to 16: the multiplier (2^32 + M0lo) / 2^32 is split into 217 / 128
@@ -390,7 +391,9 @@ __device__ __forceinline__ void cipher_inverse_items_fixed(uint32_t (&left)[ITEM
 // floor (the first one's value is rounded to a grid that holds the multiples of
 // 2^-7 at which the second one's floor steps).  The forward round gains nothing
 // from this (its product gives the low word too).  MIXED: at most 12 bits, one
-// FMA.  Measured on GB300, 2^28 evaluations at k = 28: 1.35 -> 1.15 ms.
+// FMA.  Measured on GB300, 2^28 evaluations at k = 28: 1.35 -> 1.15 ms; the shuffle of 2^27 4-byte elements
+// (odd k) 1.80 -> 1.71 ms, of 2^27 - 5 8-byte ones 2.38 -> 2.32.  Where pass 1
+// of a shuffle waits more than it computes (n over 2 GiB) nothing changes.
 constexpr float kFracTop = 217.0f / 128.0f;
 constexpr float kFracRest = -(static_cast<float>(0xB2000000u - kM0Lo) / 4294967296.0f);
 static_assert(0xB2000000u - kM0Lo < (1u << 22), "the rest of the multiplier is exact in a float");
@@ -411,7 +414,7 @@ __device__ __forceinline__ void floor_fma_onto_items(uint32_t (&d)[ITEMS], const
             : "r"(x[j]), "r"(x[j + 1]), "r"(m));
 }
 
-template <bool MIXED, int ITEMS, int ROUNDS>
+template <bool ODD, bool MIXED, int ITEMS, int ROUNDS>
 __device__ __forceinline__ void cipher_inverse_items_float(uint32_t (&left)[ITEMS], uint32_t (&right)[ITEMS],
                                                            const uint32_t *keys, const Geometry &g)
 {
@@ -422,7 +425,8 @@ __device__ __forceinline__ void cipher_inverse_items_float(uint32_t (&left)[ITEM
         const uint32_t key = keys[r];
         uint32_t old_left[ITEMS], hi[ITEMS];
 #pragma unroll
-        for (int j = 0; j < ITEMS; ++j) old_left[j] = ((right[j] * kM0InvLo) & lmask) | kFloatBase;
+        for (int j = 0; j < ITEMS; ++j)
+            old_left[j] = (((ODD ? right[j] >> 1 : right[j]) * kM0InvLo) & lmask) | kFloatBase;
         if constexpr (MIXED) {
             floor_fma_items(hi, old_left, kMixedFrac, frac_add);
         } else {
@@ -431,7 +435,8 @@ __device__ __forceinline__ void cipher_inverse_items_float(uint32_t (&left)[ITEM
         }
 #pragma unroll
         for (int j = 0; j < ITEMS; ++j) {
-            right[j] = left[j] ^ (old_left[j] * (kM0Hi - 1u) + hi[j]) ^ key;  // don't-care above bit L
+            const uint32_t x = left[j] ^ (old_left[j] * (kM0Hi - 1u) + hi[j]) ^ key;  // don't-care above bit L
+            right[j] = ODD ? ((x & lmask) | ((right[j] * g.lift_mul) & ~lmask)) : x;
             left[j] = old_left[j];
         }
     }
@@ -448,10 +453,7 @@ __device__ __forceinline__ void cipher_inverse_items(uint32_t (&left)[ITEMS], ui
                                                      const uint32_t *keys, uint32_t rounds, const Geometry &g)
 {
     if (rounds == kUnrolledRounds) {
-        if constexpr (ODD)
-            cipher_inverse_items_fixed<ODD, ITEMS, kUnrolledRounds>(left, right, keys, g);
-        else
-            cipher_inverse_items_float<FORM == CipherForm::Mixed, ITEMS, kUnrolledRounds>(left, right, keys, g);
+        cipher_inverse_items_float<ODD, FORM == CipherForm::Mixed, ITEMS, kUnrolledRounds>(left, right, keys, g);
     } else
         cipher_inverse_items_loop<ODD, ITEMS>(left, right, keys, rounds, g);
 }

@@ -196,7 +196,7 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     }
 }
 
-// FORM: Mixed or Wide (the inverse cipher's odd-k round has one form).
+// FORM: Mixed or Wide.
 template <class T, bool ODD, bool FORWARD, int ITEMS, CipherForm FORM = CipherForm::Wide>
 __global__ void __launch_bounds__(kP1Block) staged_bucket_kernel(const __grid_constant__ StagedArgs a)
 {
@@ -637,7 +637,7 @@ cudaError_t launch_p1(const StagedArgs &a, int device, cudaStream_t stream)
         even = staged_bucket_kernel<T, false, FORWARD, ITEMS>;
         if constexpr (ITEMS == 8)  // 16 items: over 2^26 elements
             if (cipher_form(a.g) != CipherForm::Wide) {
-                if constexpr (FORWARD) odd = staged_bucket_kernel<T, true, FORWARD, ITEMS, CipherForm::Mixed>;
+                odd = staged_bucket_kernel<T, true, FORWARD, ITEMS, CipherForm::Mixed>;
                 even = staged_bucket_kernel<T, false, FORWARD, ITEMS, CipherForm::Mixed>;
                 form = 1;
             }
