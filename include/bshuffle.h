@@ -351,7 +351,7 @@ int bshuffle_release_workspaces(void);
  *       so element b belongs in slot f^-1(b) (the inverse cipher of Sec. 3.2;
  *       bshuffle_inverse uses the same passes with slot f(b)).
  *       Pass 1 reads the input sequentially, inverts the cipher and buckets
- *       (value, slot) by 8 MiB output window; pass 2 scatters each window
+ *       (value, slot) by output window of 4 MiB or more; pass 2 scatters each window
  *       while it is resident in L2.  Random HBM accesses are rate-limited on
  *       GB300, streaming ones are not.  Workspace n * (4 + elem_bytes) bytes
  *       plus a little, allocated on first use per stream.  Other n (the
@@ -369,8 +369,9 @@ int bshuffle_release_workspaces(void);
  *       16-byte elements and for indices (rows run the plain single pass):
  *       persistent CTAs; eight compute warps evaluate the bijection of a tile
  *       and copy its kept elements into shared memory with cp.async (1- and
- *       2-byte elements are read when they are stored), then store the previous tile, which a ninth warp has meanwhile ranked
- *       with the look-back.  Same memory traffic and workspace as the single
+ *       2-byte elements are read when they are stored), then store the
+ *       previous tile, which a ninth warp has meanwhile ranked with the
+ *       look-back.  Same memory traffic and workspace as the single
  *       pass.
  *   BSHUFFLE_STRATEGY_AUTO (default)  staged when it applies and
  *       n * elem_bytes >= 256 MiB (for n other than 2^k: with 4- or 8-byte

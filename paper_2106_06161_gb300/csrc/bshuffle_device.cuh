@@ -392,8 +392,7 @@ __device__ __forceinline__ void cipher_inverse_items_fixed(uint32_t (&left)[ITEM
 // 2^-7 at which the second one's floor steps).  The forward round gains nothing
 // from this (its product gives the low word too).  MIXED: at most 12 bits, one
 // FMA.  Measured on GB300, 2^28 evaluations at k = 28: 1.35 -> 1.15 ms; the shuffle of 2^27 4-byte elements
-// (odd k) 1.80 -> 1.71 ms, of 2^27 - 5 8-byte ones 2.38 -> 2.32.  Where pass 1
-// of a shuffle waits more than it computes (n over 2 GiB) nothing changes.
+// (odd k) 1.80 -> 1.71 ms, of 2^27 - 5 8-byte ones 2.38 -> 2.32.
 constexpr float kFracTop = 217.0f / 128.0f;
 constexpr float kFracRest = -(static_cast<float>(0xB2000000u - kM0Lo) / 4294967296.0f);
 static_assert(0xB2000000u - kM0Lo < (1u << 22), "the rest of the multiplier is exact in a float");

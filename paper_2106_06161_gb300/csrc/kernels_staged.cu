@@ -35,9 +35,9 @@
 // P1 slows down steeply past 256 buckets per 2,048-element chunk (each chunk
 // zeroes, scans and atomically appends every bucket).  staged_window_shift
 // takes the smallest window (at least 4 MiB) that keeps the bucket count at
-// one per 8 elements of a P1 chunk, and inputs over 2 GiB of 4- or 8-byte
-// elements use 4,096-element chunks (16 items per thread), which halves the
-// appends per element and allows 512 buckets.
+// one per 8 elements of a P1 chunk, and inputs from 1 GiB on of 4- or 8-byte
+// elements use 4,096-element chunks (512 threads), which halves the appends per
+// element and allows 512 buckets.
 //
 // Ranked form (n not a power of two, domain 2^k > n): element b still goes to
 // the slot of its domain index i = f^-1(b), but that slot is the rank of i
@@ -63,31 +63,37 @@ using dev::kFull;
 constexpr int kSBlock = 256;
 constexpr int kSItems = 8;
 constexpr uint32_t kSTile = kSBlock * kSItems;  // entries per CTA of P2
-// P1's CTA size (overridable at build time for tuning experiments): a P1 CTA
-// buckets kP1Block * ITEMS consecutive elements, ITEMS = 8 or 16.
-#ifndef BSHUFFLE_STAGED_P1_BLOCK
-#define BSHUFFLE_STAGED_P1_BLOCK 256
-#endif
-constexpr int kP1Block = BSHUFFLE_STAGED_P1_BLOCK;
-constexpr int kP1Warps = kP1Block / 32;
-constexpr uint32_t kP1TileSmall = kP1Block * 8;
-constexpr uint32_t kP1TileLarge = kP1Block * 16;
+// A P1 CTA buckets a chunk of kP1Items consecutive elements per thread, with
+// 256 threads or 512.  (The large chunk with 16 items in 256 threads takes 80
+// registers and more, so 24 warps per SM at most instead of 32 or 48, too few to
+// hide the pass's steps: uint64 shuffle of 2^28 + 12345 elements 5.03 -> 4.81 ms,
+// its inverse 8.47 -> 7.56, the shuffle of 2^29 8.72 -> 8.30.)
+constexpr int kP1Items = 8;
+constexpr int kP1Small = 256;
+constexpr int kP1Large = 512;
+constexpr uint32_t kP1TileSmall = kP1Small * kP1Items;
+constexpr uint32_t kP1TileLarge = kP1Large * kP1Items;
 constexpr uint32_t kStagedMinChunk = kP1TileSmall > kSTile ? kP1TileSmall : kSTile;
 constexpr uint32_t kMinWindowLog2 = 22;       // 4 MiB
-constexpr uint64_t kLargeInputBytes = uint64_t{1} << 31;  // above this, 16 items per P1 thread
+// From here on P1 takes the large chunk: uint64 shuffles of 2^27, small and
+// large, 1.91 and 1.88 ms, of 2^28 3.63 and 3.43, of 2^28 - 5 4.43 and 4.31, its
+// inverse 4.91 and 4.77; uint32 of 2^28 3.03 and 2.96.  At half of it the two are
+// level (uint64 of 2^26 + 1 1.161 and 1.166, uint32 of 2^27 1.704 and 1.714).
+constexpr uint64_t kLargeInputBytes = uint64_t{1} << 30;
 
-// P1 items per thread for n elements of elem_bytes.
-uint32_t p1_items_for(uint64_t n, uint32_t elem_bytes)
+// P1 threads per CTA for n elements of elem_bytes.
+int p1_threads_for(uint64_t n, uint32_t elem_bytes)
 {
-    return elem_bytes <= 8 && n * elem_bytes > kLargeInputBytes ? 16u : 8u;
+    return elem_bytes <= 8 && n * elem_bytes >= kLargeInputBytes ? kP1Large : kP1Small;
 }
 
-// Exclusive scan of cnt[0..m) into start[0..m) by the whole CTA (kP1Block threads).
+// Exclusive scan of cnt[0..m) into start[0..m) by the whole CTA (BLOCK threads).
+template <int BLOCK>
 __device__ __forceinline__ void block_exclusive_scan(const uint32_t *cnt, uint32_t *start, uint32_t m,
                                                      uint32_t *s_warp)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const uint32_t per = (m + kP1Block - 1) / kP1Block;
+    const uint32_t per = (m + BLOCK - 1) / BLOCK;
     const uint32_t b0 = tid * per;
     const uint32_t b1 = b0 + per < m ? b0 + per : m;
     uint32_t sum = 0;
@@ -96,9 +102,9 @@ __device__ __forceinline__ void block_exclusive_scan(const uint32_t *cnt, uint32
     if (lane == 31) s_warp[warp] = incl;
     __syncthreads();
     if (warp == 0) {
-        const uint32_t w = lane < static_cast<uint32_t>(kP1Warps) ? s_warp[lane] : 0u;
+        const uint32_t w = lane < BLOCK / 32u ? s_warp[lane] : 0u;
         const uint32_t wi = dev::warp_inclusive_scan(w);
-        if (lane < static_cast<uint32_t>(kP1Warps)) s_warp[lane] = wi - w;
+        if (lane < BLOCK / 32u) s_warp[lane] = wi - w;
     }
     __syncthreads();
     uint32_t run = s_warp[warp] + incl - sum;
@@ -115,11 +121,10 @@ __device__ __forceinline__ void block_exclusive_scan(const uint32_t *cnt, uint32
 // bucket is a window of domain indices and the last chunk is ragged.  The
 // round keys sit in kernel parameter space, so the unrolled 24 rounds read
 // them as constant operands.
-template <class T, bool ODD, bool FORWARD, int ITEMS, bool PADDED, CipherForm FORM = CipherForm::Wide>
+template <class T, bool ODD, bool FORWARD, int BLOCK, bool PADDED, CipherForm FORM = CipherForm::Wide>
 __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
 {
-    constexpr int kP1Items = ITEMS;
-    constexpr uint32_t kP1Tile = kP1Block * ITEMS;
+    constexpr uint32_t kP1Tile = BLOCK * kP1Items;
     // dynamic shared memory: the chunk's entries (value, output slot) sorted
     // by destination bucket, then three words per destination bucket.  The
     // bucket and the entry's staged offset are recomputed from the slot at
@@ -131,7 +136,7 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_raw + kP1Tile * (sizeof(T) + 4));
     uint32_t *s_start = s_cnt + a.num_dst;
     uint32_t *s_gbase = s_start + a.num_dst;
-    __shared__ uint32_t s_warp[kP1Warps];
+    __shared__ uint32_t s_warp[BLOCK / 32];
 
     const uint32_t tid = threadIdx.x;
     const Geometry &g = a.g;
@@ -139,19 +144,19 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     const uint32_t first = blockIdx.x * kP1Tile;
     const uint32_t chunk = PADDED ? min(kP1Tile, g.n - first) : kP1Tile;
     const T *in = static_cast<const T *>(a.in);
-    for (uint32_t q = tid; q < a.num_dst; q += kP1Block) s_cnt[q] = 0u;
+    for (uint32_t q = tid; q < a.num_dst; q += BLOCK) s_cnt[q] = 0u;
 
     T val[kP1Items];
     uint32_t left[kP1Items], right[kP1Items];
 #pragma unroll
     for (int j = 0; j < kP1Items; ++j) {
-        const uint32_t b = first + static_cast<uint32_t>(j * kP1Block) + tid;
+        const uint32_t b = first + static_cast<uint32_t>(j * BLOCK) + tid;
         if (!PADDED || b < g.n) val[j] = __ldcs(in + b);
         if (!FORWARD) left[j] = b >> g.R;  // beyond a padded n: never used
         if (!FORWARD) right[j] = b & g.rmask;
     }
     if constexpr (FORWARD)
-        dev::cipher_run_wide<ODD, kP1Items, kP1Block, FORM>(left, right, first + tid, a.keys, a.rounds, g);
+        dev::cipher_run_wide<ODD, kP1Items, BLOCK, FORM>(left, right, first + tid, a.keys, a.rounds, g);
     else
         dev::cipher_inverse_items<ODD, kP1Items, FORM>(left, right, a.keys, a.rounds, g);
     uint32_t dst[kP1Items], slot[kP1Items];
@@ -160,18 +165,18 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     __syncthreads();  // s_cnt zeroed
 #pragma unroll
     for (int j = 0; j < kP1Items; ++j)
-        if (!PADDED || static_cast<uint32_t>(j * kP1Block) + tid < chunk)
+        if (!PADDED || static_cast<uint32_t>(j * BLOCK) + tid < chunk)
             slot[j] = atomicAdd(&s_cnt[dst[j] >> a.dst_shift], 1u);
     __syncthreads();
-    block_exclusive_scan(s_cnt, s_start, a.num_dst, s_warp);
-    for (uint32_t q = tid; q < a.num_dst; q += kP1Block) {
+    block_exclusive_scan<BLOCK>(s_cnt, s_start, a.num_dst, s_warp);
+    for (uint32_t q = tid; q < a.num_dst; q += BLOCK) {
         const uint32_t c = s_cnt[q];
         s_gbase[q] = c != 0u ? atomicAdd(&a.dst_cursor[q], c) : 0u;
     }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kP1Items; ++j) {
-        if (PADDED && static_cast<uint32_t>(j * kP1Block) + tid >= chunk) continue;
+        if (PADDED && static_cast<uint32_t>(j * BLOCK) + tid >= chunk) continue;
         const uint32_t p = s_start[dst[j] >> a.dst_shift] + slot[j];
         s_val[p] = val[j];
         s_dst[p] = dst[j];
@@ -181,7 +186,7 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
     const uint32_t bmask = static_cast<uint32_t>((uint64_t{1} << a.dst_shift) - 1u);
 #pragma unroll
     for (int j = 0; j < kP1Items; ++j) {
-        const uint32_t p = static_cast<uint32_t>(j * kP1Block) + tid;
+        const uint32_t p = static_cast<uint32_t>(j * BLOCK) + tid;
         if (PADDED && p >= chunk) continue;
         const uint32_t d = s_dst[p];
         const uint32_t q = static_cast<uint32_t>(static_cast<uint64_t>(d) >> a.dst_shift);
@@ -197,32 +202,36 @@ __device__ __forceinline__ void bucket_pass(const StagedArgs &a)
 }
 
 // FORM: Mixed or Wide.
-template <class T, bool ODD, bool FORWARD, int ITEMS, CipherForm FORM = CipherForm::Wide>
-__global__ void __launch_bounds__(kP1Block) staged_bucket_kernel(const __grid_constant__ StagedArgs a)
+template <class T, bool ODD, bool FORWARD, int BLOCK, CipherForm FORM = CipherForm::Wide>
+__global__ void __launch_bounds__(BLOCK) staged_bucket_kernel(const __grid_constant__ StagedArgs a)
 {
-    bucket_pass<T, ODD, FORWARD, ITEMS, false, FORM>(a);
+    bucket_pass<T, ODD, FORWARD, BLOCK, false, FORM>(a);
+}
+
+// The large chunk with the forward cipher (the inverse shuffle): three CTAs per
+// SM instead of the two that the compiler's own choice allows.  Inverse of
+// 2^28 8-byte elements 3.57 -> 3.46 ms, of 2^29 8.06 -> 7.85; with the inverse
+// cipher the same cap spills and costs 2 % (2^28 3.50 -> 3.59).
+template <class T, bool ODD>
+__global__ void __launch_bounds__(kP1Large, 3) staged_bucket_forward_large_kernel(const __grid_constant__ StagedArgs a)
+{
+    bucket_pass<T, ODD, true, kP1Large, false, CipherForm::Wide>(a);
 }
 
 // The ranked form's P1, in kernels of its own so that their register
-// budgets are set apart from the 2^k form's.  With 16 items per thread and
-// 4- or 8-byte elements the compiler would take 92-94 registers (2 CTAs per
-// SM); capped for 3 CTAs per SM, pass 1 of the n = 2^28 + 12345 uint64
-// shuffle takes 2.61 ms instead of 2.85 ms on GB300 (16-byte elements spill
-// under the cap and keep 2 CTAs).
-template <class T, bool ODD, int ITEMS>
-__global__ void __launch_bounds__(kP1Block) staged_rank_bucket_kernel(const __grid_constant__ StagedArgs a)
+// budgets are set apart from the 2^k form's: with the large chunk three CTAs
+// per SM (42 registers) gain for 4-byte elements (n = 2^28 + 12345 4.54 -> 4.45
+// ms in all, 8-byte ones 4.81 either way; 16-byte elements would spill).
+template <class T, bool ODD, int BLOCK>
+__global__ void __launch_bounds__(BLOCK) staged_rank_bucket_kernel(const __grid_constant__ StagedArgs a)
 {
-    bucket_pass<T, ODD, false, ITEMS, true>(a);
+    bucket_pass<T, ODD, false, BLOCK, true>(a);
 }
 
-#ifndef BSHUFFLE_RANKED_P1_MIN_CTAS
-#define BSHUFFLE_RANKED_P1_MIN_CTAS 3
-#endif
 template <class T, bool ODD>
-__global__ void __launch_bounds__(kP1Block, BSHUFFLE_RANKED_P1_MIN_CTAS)
-    staged_rank_bucket16_kernel(const __grid_constant__ StagedArgs a)
+__global__ void __launch_bounds__(kP1Large, 3) staged_rank_bucket_large_kernel(const __grid_constant__ StagedArgs a)
 {
-    bucket_pass<T, ODD, false, 16, true>(a);
+    bucket_pass<T, ODD, false, kP1Large, true>(a);
 }
 
 // The inverse shuffle's P1 for n < 2^k: out[f(i_j)] = in[j].  A CTA owns a
@@ -240,18 +249,19 @@ __global__ void __launch_bounds__(kP1Block, BSHUFFLE_RANKED_P1_MIN_CTAS)
 // pass is bound by the cipher over the whole domain (the odd-k forward round)
 // and waits on the look-back: publishing the count before the window counts
 // took 2^28 + 12345 uint64 from 8.93 to 8.65 ms (single pass 10.7).
-template <class T, bool ODD, int ITEMS, CipherForm FORM>
-__global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const __grid_constant__ StagedArgs a)
+template <class T, bool ODD, int BLOCK, CipherForm FORM>
+__global__ void __launch_bounds__(BLOCK) staged_inverse_bucket_kernel(const __grid_constant__ StagedArgs a)
 {
-    constexpr uint32_t kTile = kP1Block * ITEMS;
+    constexpr int ITEMS = kP1Items, WARPS = BLOCK / 32;
+    constexpr uint32_t kTile = BLOCK * ITEMS;
     extern __shared__ __align__(16) unsigned char s_raw[];
     T *s_val = reinterpret_cast<T *>(s_raw);
     uint32_t *s_dst = reinterpret_cast<uint32_t *>(s_raw + kTile * sizeof(T));
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_raw + kTile * (sizeof(T) + 4));
     uint32_t *s_start = s_cnt + a.num_dst;
     uint32_t *s_gbase = s_start + a.num_dst;
-    __shared__ dev::TileShared<ITEMS * kP1Warps> st;
-    __shared__ uint32_t s_warp[kP1Warps];
+    __shared__ dev::TileShared<ITEMS * WARPS> st;
+    __shared__ uint32_t s_warp[WARPS];
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const Geometry &g = a.g;
@@ -259,7 +269,7 @@ __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const _
         st.tile = atomicAdd(&a.ws->ticket, 1u);
         st.tag = dev::ld_relaxed_gpu(&a.ws->tag);
     }
-    for (uint32_t q = tid; q < a.num_dst; q += kP1Block) s_cnt[q] = 0u;
+    for (uint32_t q = tid; q < a.num_dst; q += BLOCK) s_cnt[q] = 0u;
     __syncthreads();
     const uint32_t tile = st.tile, tag = st.tag;
     if (tile >= a.num_tiles) {  // only a corrupted header could hand out such a ticket
@@ -272,18 +282,18 @@ __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const _
     // the domain is a multiple of the chunk
     const uint32_t base = tile * kTile + tid;
     uint32_t left[ITEMS], right[ITEMS];
-    dev::cipher_run_wide<ODD, ITEMS, kP1Block, FORM>(left, right, base, a.keys, a.rounds, g);
+    dev::cipher_run_wide<ODD, ITEMS, BLOCK, FORM>(left, right, base, a.keys, a.rounds, g);
     uint32_t dst[ITEMS], mask[ITEMS], slot[ITEMS];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
         dst[j] = (left[j] << g.R) | right[j];
         mask[j] = __ballot_sync(kFull, dst[j] < g.n);
-        if (lane == 0) st.counts[j * kP1Warps + warp] = static_cast<uint32_t>(__popc(mask[j]));
+        if (lane == 0) st.counts[j * WARPS + warp] = static_cast<uint32_t>(__popc(mask[j]));
     }
     __syncthreads();
     // the last warp publishes the chunk's count before anything else: later
     // chunks wait for it
-    const bool ranker = warp == kP1Warps - 1;
+    const bool ranker = warp == WARPS - 1;
     const dev::StatusRing ring{a.status, ~0ull, 63u, tag};
     uint32_t aggregate = 0;
     if (ranker) aggregate = dev::tile_scan_publish(st, ring, tile, 0, a.skip_publish_tile);
@@ -295,12 +305,12 @@ __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const _
     if (ranker) {
         dev::tile_lookback(st, aggregate, ring, tile, 0, a.timeout_ns, a.skip_publish_tile, a.ws);
     } else {
-        for (uint32_t q = tid; q < a.num_dst; q += kP1Block - 32u) {
+        for (uint32_t q = tid; q < a.num_dst; q += BLOCK - 32u) {
             const uint32_t c = s_cnt[q];
             s_gbase[q] = c != 0u ? atomicAdd(&a.dst_cursor[q], c) : 0u;
         }
     }
-    block_exclusive_scan(s_cnt, s_start, a.num_dst, s_warp);
+    block_exclusive_scan<BLOCK>(s_cnt, s_start, a.num_dst, s_warp);
     __syncthreads();
     // an unranked chunk (the look-back ran out of time) moves zeros: its
     // window entries have to be there for the next pass
@@ -312,7 +322,7 @@ __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const _
     for (int j = 0; j < ITEMS; ++j) {
         val[j] = T{};
         if (dst[j] >= g.n) continue;
-        const uint32_t src = prefix + st.counts[j * kP1Warps + warp] + static_cast<uint32_t>(__popc(mask[j] & lt));
+        const uint32_t src = prefix + st.counts[j * WARPS + warp] + static_cast<uint32_t>(__popc(mask[j] & lt));
         if (ok && src < g.n) val[j] = __ldcs(in + src);
         else if (ok) dev::record_error(a.ws, dev::kErrDeviceBounds, src);
     }
@@ -329,7 +339,7 @@ __global__ void __launch_bounds__(kP1Block) staged_inverse_bucket_kernel(const _
     const uint32_t kept = st.aggregate;
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t p = static_cast<uint32_t>(j * kP1Block) + tid;
+        const uint32_t p = static_cast<uint32_t>(j * BLOCK) + tid;
         if (p >= kept) continue;
         const uint32_t d = s_dst[p];
         const uint32_t q = d >> a.dst_shift;
@@ -410,11 +420,9 @@ constexpr uint32_t kRankMaxSubShift = 20;
 constexpr uint32_t kSuperWords = 2048;  // bitmap words per 32-bit prefix (2^16 indices)
 constexpr int kRankUnroll = 4;          // uint4 loads of 4 offsets each, per thread and step
 constexpr uint32_t kRanked = 0x80000000u;
-// The ranked form takes 16 P1 items per thread (512 buckets) where 8 would
-// leave spans over 2^BSHUFFLE_RANKED_MAX_SPAN_LOG2 domain indices.
-#ifndef BSHUFFLE_RANKED_MAX_SPAN_LOG2
-#define BSHUFFLE_RANKED_MAX_SPAN_LOG2 20
-#endif
+// The ranked form takes P1's large chunk (512 buckets) where the small one
+// would leave spans over 2^kRankedMaxSpanLog2 domain indices.
+constexpr uint32_t kRankedMaxSpanLog2 = 20;
 
 size_t rank_smem_bytes(uint32_t sub_shift)
 {
@@ -607,10 +615,10 @@ __global__ void __launch_bounds__(kSBlock) staged_rank_scatter_kernel(const __gr
 }
 
 // P1's dynamic shared memory for num_dst destination buckets.
-template <class T, int ITEMS>
+template <class T, int BLOCK>
 constexpr size_t p1_smem_bytes(uint32_t num_dst)
 {
-    return size_t{kP1Block} * ITEMS * (sizeof(T) + sizeof(uint32_t)) + 3u * num_dst * sizeof(uint32_t);
+    return size_t{BLOCK} * kP1Items * (sizeof(T) + sizeof(uint32_t)) + 3u * num_dst * sizeof(uint32_t);
 }
 
 cudaError_t mark(cudaEvent_t *marks, int i, cudaStream_t stream)
@@ -618,42 +626,45 @@ cudaError_t mark(cudaEvent_t *marks, int i, cudaStream_t stream)
     return marks != nullptr ? cudaEventRecord(marks[i], stream) : cudaSuccess;
 }
 
-// P1 with ITEMS per thread: the odd and even instances, each allowed the
+// P1 with BLOCK threads: the odd and even instances, each allowed the
 // shared memory of 4096 buckets on first use on a device.
-template <class T, bool FORWARD, int ITEMS, bool PADDED>
+template <class T, bool FORWARD, int BLOCK, bool PADDED>
 cudaError_t launch_p1(const StagedArgs &a, int device, cudaStream_t stream)
 {
     using Kernel = void (*)(StagedArgs);
     Kernel odd, even;
     int form = 0;
-    if constexpr (PADDED && ITEMS == 16 && sizeof(T) <= 8) {
-        odd = staged_rank_bucket16_kernel<T, true>;
-        even = staged_rank_bucket16_kernel<T, false>;
+    if constexpr (PADDED && BLOCK == kP1Large && sizeof(T) <= 8) {
+        odd = staged_rank_bucket_large_kernel<T, true>;
+        even = staged_rank_bucket_large_kernel<T, false>;
     } else if constexpr (PADDED) {
-        odd = staged_rank_bucket_kernel<T, true, ITEMS>;
-        even = staged_rank_bucket_kernel<T, false, ITEMS>;
+        odd = staged_rank_bucket_kernel<T, true, BLOCK>;
+        even = staged_rank_bucket_kernel<T, false, BLOCK>;
+    } else if constexpr (FORWARD && BLOCK == kP1Large) {
+        odd = staged_bucket_forward_large_kernel<T, true>;
+        even = staged_bucket_forward_large_kernel<T, false>;
     } else {
-        odd = staged_bucket_kernel<T, true, FORWARD, ITEMS>;
-        even = staged_bucket_kernel<T, false, FORWARD, ITEMS>;
-        if constexpr (ITEMS == 8)  // 16 items: over 2^26 elements
+        odd = staged_bucket_kernel<T, true, FORWARD, BLOCK>;
+        even = staged_bucket_kernel<T, false, FORWARD, BLOCK>;
+        if constexpr (BLOCK == kP1Small)  // the large one: from 2^27 elements on
             if (cipher_form(a.g) != CipherForm::Wide) {
-                odd = staged_bucket_kernel<T, true, FORWARD, ITEMS, CipherForm::Mixed>;
-                even = staged_bucket_kernel<T, false, FORWARD, ITEMS, CipherForm::Mixed>;
+                odd = staged_bucket_kernel<T, true, FORWARD, BLOCK, CipherForm::Mixed>;
+                even = staged_bucket_kernel<T, false, FORWARD, BLOCK, CipherForm::Mixed>;
                 form = 1;
             }
     }
     static std::atomic<bool> configured[2][64];  // attribute set on this device
     if (!configured[form][device].load(std::memory_order_acquire)) {
-        const int most = static_cast<int>(p1_smem_bytes<T, ITEMS>(4096));
+        const int most = static_cast<int>(p1_smem_bytes<T, BLOCK>(4096));
         cudaError_t e = cudaFuncSetAttribute(odd, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(even, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
         configured[form][device].store(true, std::memory_order_release);
     }
-    const size_t dyn = p1_smem_bytes<T, ITEMS>(a.num_dst);
-    const uint64_t tile = uint64_t{kP1Block} * ITEMS;
+    const size_t dyn = p1_smem_bytes<T, BLOCK>(a.num_dst);
+    const uint64_t tile = uint64_t{BLOCK} * kP1Items;
     const unsigned chunks = static_cast<unsigned>((static_cast<uint64_t>(a.g.n) + tile - 1) / tile);
-    ((a.g.k & 1u) ? odd : even)<<<chunks, kP1Block, dyn, stream>>>(a);
+    ((a.g.k & 1u) ? odd : even)<<<chunks, BLOCK, dyn, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -702,25 +713,25 @@ cudaError_t launch_rank(const StagedArgs &a, int device, cudaStream_t stream)
 
 
 // P1 of the inverse shuffle for n < 2^k.
-template <class T, int ITEMS, CipherForm FORM>
+template <class T, int BLOCK, CipherForm FORM>
 cudaError_t launch_inverse_p1(const StagedArgs &a, int device, cudaStream_t stream)
 {
-    const auto odd = staged_inverse_bucket_kernel<T, true, ITEMS, FORM>;
-    const auto even = staged_inverse_bucket_kernel<T, false, ITEMS, FORM>;
+    const auto odd = staged_inverse_bucket_kernel<T, true, BLOCK, FORM>;
+    const auto even = staged_inverse_bucket_kernel<T, false, BLOCK, FORM>;
     static std::atomic<bool> configured[64];  // attribute set on this device
     if (!configured[device].load(std::memory_order_acquire)) {
-        const int most = static_cast<int>(p1_smem_bytes<T, ITEMS>(4096));
+        const int most = static_cast<int>(p1_smem_bytes<T, BLOCK>(4096));
         cudaError_t e = cudaFuncSetAttribute(odd, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(even, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e != cudaSuccess) return e;
         configured[device].store(true, std::memory_order_release);
     }
-    ((a.g.k & 1u) ? odd : even)<<<a.num_tiles, kP1Block, p1_smem_bytes<T, ITEMS>(a.num_dst), stream>>>(a);
+    ((a.g.k & 1u) ? odd : even)<<<a.num_tiles, BLOCK, p1_smem_bytes<T, BLOCK>(a.num_dst), stream>>>(a);
     return cudaGetLastError();
 }
 
 template <class T, bool FORWARD>
-cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t stream, cudaEvent_t *marks)
+cudaError_t launch_typed(const StagedArgs &a, bool large, cudaStream_t stream, cudaEvent_t *marks)
 {
     static std::atomic<bool> configured[64];  // attribute set on this device
     int device = 0;
@@ -741,21 +752,21 @@ cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t strea
     if (e != cudaSuccess) return e;
     if (padded) {
         if constexpr (!FORWARD)
-            e = items == 16 ? launch_p1<T, false, 16, true>(a, device, stream)
-                            : launch_p1<T, false, 8, true>(a, device, stream);
+            e = large ? launch_p1<T, false, kP1Large, true>(a, device, stream)
+                            : launch_p1<T, false, kP1Small, true>(a, device, stream);
         else if (cipher_form(a.g) != CipherForm::Wide)
-            e = items == 16 ? cudaErrorInvalidValue  // over 2 GiB, so over 2^26 elements
-                            : launch_inverse_p1<T, 8, CipherForm::Mixed>(a, device, stream);
+            e = large ? cudaErrorInvalidValue  // from 1 GiB, so from 2^27 elements on
+                            : launch_inverse_p1<T, kP1Small, CipherForm::Mixed>(a, device, stream);
         else if constexpr (sizeof(T) <= 8)
-            e = items == 16 ? launch_inverse_p1<T, 16, CipherForm::Wide>(a, device, stream)
-                            : launch_inverse_p1<T, 8, CipherForm::Wide>(a, device, stream);
+            e = large ? launch_inverse_p1<T, kP1Large, CipherForm::Wide>(a, device, stream)
+                            : launch_inverse_p1<T, kP1Small, CipherForm::Wide>(a, device, stream);
         else
-            e = launch_inverse_p1<T, 8, CipherForm::Wide>(a, device, stream);
+            e = launch_inverse_p1<T, kP1Small, CipherForm::Wide>(a, device, stream);
     } else if constexpr (sizeof(T) <= 8) {
-        e = items == 16 ? launch_p1<T, FORWARD, 16, false>(a, device, stream)
-                        : launch_p1<T, FORWARD, 8, false>(a, device, stream);
+        e = large ? launch_p1<T, FORWARD, kP1Large, false>(a, device, stream)
+                        : launch_p1<T, FORWARD, kP1Small, false>(a, device, stream);
     } else {
-        e = launch_p1<T, FORWARD, 8, false>(a, device, stream);
+        e = launch_p1<T, FORWARD, kP1Small, false>(a, device, stream);
     }
     if (e == cudaSuccess) e = mark(marks, 1, stream);
     if (e != cudaSuccess) return e;
@@ -774,24 +785,23 @@ cudaError_t launch_typed(const StagedArgs &a, uint32_t items, cudaStream_t strea
 }
 
 // The ranked form's shape: one bucket per 8 elements of a P1 chunk (256
-// buckets with 8 items per thread, 512 with 16), spans of at least 2^12
-// indices, 16 items per thread where 8 would leave spans over 2^20 indices
+// buckets, or 512 with the large chunk), spans of at least 2^12 indices, the
+// large chunk where the small one would leave spans over 2^20 indices
 // (one CTA then ranks a whole span up to 2^29-index domains), and at most 8
 // parts of 2^20 indices per span (a portable cluster), with more buckets
 // where a span would need more parts.
 void rank_config(uint64_t n, uint32_t k, uint32_t elem_bytes, uint32_t *bucket_shift, uint32_t *sub_shift,
-                 uint32_t *items)
+                 bool *large)
 {
-    uint32_t it = p1_items_for(n, elem_bytes);
-    if (k > 8 && k - 8 > BSHUFFLE_RANKED_MAX_SPAN_LOG2) it = 16;
-    const uint32_t buckets_log2 = it == 16 ? 9u : 8u;
+    const bool big = p1_threads_for(n, elem_bytes) == kP1Large || (k > 8 && k - 8 > kRankedMaxSpanLog2);
+    const uint32_t buckets_log2 = big ? 9u : 8u;
     uint32_t s = k > buckets_log2 ? k - buckets_log2 : 0u;
     const uint32_t floor_shift = k < 12 ? k : 12u;
     if (s < floor_shift) s = floor_shift;
     if (s > kRankMaxSubShift + 3) s = kRankMaxSubShift + 3;
     *bucket_shift = s;
     *sub_shift = s < kRankMaxSubShift ? s : kRankMaxSubShift;
-    *items = it;
+    *large = big;
 }
 
 }  // namespace
@@ -800,7 +810,7 @@ uint32_t staged_tile_size() { return kStagedMinChunk; }
 
 uint32_t staged_p1_tile(uint64_t n, uint32_t elem_bytes)
 {
-    return p1_items_for(n, elem_bytes) == 16u ? kP1TileLarge : kP1TileSmall;
+    return p1_threads_for(n, elem_bytes) == kP1Large ? kP1TileLarge : kP1TileSmall;
 }
 
 uint32_t staged_window_shift(uint64_t n, uint32_t elem_bytes)
@@ -811,7 +821,7 @@ uint32_t staged_window_shift(uint64_t n, uint32_t elem_bytes)
     while ((1u << eb_log2) < elem_bytes) ++eb_log2;
     // one bucket per 8 elements of a P1 chunk: 256 (or 512) buckets
     uint32_t bucket_log2 = 0;
-    while ((8u << bucket_log2) < static_cast<uint32_t>(kP1Block) * p1_items_for(n, elem_bytes)) ++bucket_log2;
+    while ((8u << bucket_log2) < staged_p1_tile(n, elem_bytes)) ++bucket_log2;
     uint32_t shift = lg > bucket_log2 ? lg - bucket_log2 : 0u;
     const uint32_t min_shift = kMinWindowLog2 > eb_log2 ? kMinWindowLog2 - eb_log2 : 0u;
     if (shift < min_shift) shift = min_shift;
@@ -822,16 +832,16 @@ uint32_t staged_window_shift(uint64_t n, uint32_t elem_bytes)
 
 void staged_rank_shifts(uint64_t n, uint32_t k, uint32_t elem_bytes, uint32_t *bucket_shift, uint32_t *sub_shift)
 {
-    uint32_t items = 0;
-    rank_config(n, k, elem_bytes, bucket_shift, sub_shift, &items);
+    bool large = false;
+    rank_config(n, k, elem_bytes, bucket_shift, sub_shift, &large);
 }
 
 
 cudaError_t launch_staged(const StagedArgs &a, uint32_t elem_bytes, bool inverse, cudaStream_t stream,
                           cudaEvent_t *marks)
 {
-    uint32_t items = p1_items_for(a.g.n, elem_bytes);
-    const uint64_t p1_tile = items == 16 ? kP1TileLarge : kP1TileSmall;
+    bool large = p1_threads_for(a.g.n, elem_bytes) == kP1Large;
+    const uint64_t p1_tile = large ? kP1TileLarge : kP1TileSmall;
     if (static_cast<uint64_t>(a.g.n) != a.g.domain && inverse) {
         if (a.num_dst > 4096 || a.g.domain < 2 * kStagedMinChunk || a.g.domain > (uint64_t{1} << 32) ||
             a.g.domain != uint64_t{a.num_tiles} * p1_tile || a.dst_shift >= 32u ||
@@ -840,7 +850,7 @@ cudaError_t launch_staged(const StagedArgs &a, uint32_t elem_bytes, bool inverse
     } else if (static_cast<uint64_t>(a.g.n) != a.g.domain) {
         // ranked form: any n below its 2^k domain
         uint32_t s = 0, w = 0;
-        rank_config(a.g.n, a.g.k, elem_bytes, &s, &w, &items);
+        rank_config(a.g.n, a.g.k, elem_bytes, &s, &w, &large);
         if (a.g.n == 0 || a.g.domain > (uint64_t{1} << 32) || a.dst_shift != s || a.sub_shift != w ||
             (static_cast<uint64_t>(a.num_dst) << a.dst_shift) != a.g.domain || a.num_dst > 4096)
             return cudaErrorInvalidValue;
@@ -850,12 +860,12 @@ cudaError_t launch_staged(const StagedArgs &a, uint32_t elem_bytes, bool inverse
         return cudaErrorInvalidValue;
     }
     switch (elem_bytes) {
-    case 4: return inverse ? launch_typed<unsigned int, true>(a, items, stream, marks)
-                           : launch_typed<unsigned int, false>(a, items, stream, marks);
-    case 8: return inverse ? launch_typed<unsigned long long, true>(a, items, stream, marks)
-                           : launch_typed<unsigned long long, false>(a, items, stream, marks);
-    case 16: return inverse ? launch_typed<uint4, true>(a, items, stream, marks)
-                            : launch_typed<uint4, false>(a, items, stream, marks);
+    case 4: return inverse ? launch_typed<unsigned int, true>(a, large, stream, marks)
+                           : launch_typed<unsigned int, false>(a, large, stream, marks);
+    case 8: return inverse ? launch_typed<unsigned long long, true>(a, large, stream, marks)
+                           : launch_typed<unsigned long long, false>(a, large, stream, marks);
+    case 16: return inverse ? launch_typed<uint4, true>(a, large, stream, marks)
+                            : launch_typed<uint4, false>(a, large, stream, marks);
     default: return cudaErrorInvalidValue;
     }
 }
