@@ -229,10 +229,10 @@ def packed_descs(data: torch.Tensor, out: torch.Tensor, sizes, seeds) -> torch.T
     if not data.is_contiguous() or not out.is_contiguous() or out.shape != data.shape:
         raise ValueError("data and out must be contiguous tensors of one shape")
     sizes = np.asarray(sizes, dtype=np.int64)
-    if sizes.sum() != data.shape[0]:
+    ends = np.cumsum(sizes)
+    if (int(ends[-1]) if ends.size else 0) != data.shape[0]:
         raise ValueError("sizes must add up to len(data)")
-    eb = row_bytes(data)
-    offsets = np.concatenate([[0], np.cumsum(sizes)[:-1]]).astype(np.uint64) * np.uint64(eb)
+    offsets = (ends - sizes).astype(np.uint64) * np.uint64(row_bytes(data))
     return _descs(np.uint64(data.data_ptr()) + offsets, np.uint64(out.data_ptr()) + offsets, sizes,
                   list(seeds), data.device)
 
