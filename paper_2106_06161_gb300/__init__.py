@@ -164,7 +164,8 @@ def indices(n: int, seed: int, rounds: int = DEFAULT_ROUNDS, dtype: torch.dtype 
 
 
 def _descs(in_ptrs, out_ptrs, sizes, seeds, device) -> torch.Tensor:
-    """Device array of bshuffle_desc {in, out, n, seed} as int64 words."""
+    """Device array of bshuffle_desc {in, out, n, seed} as int64 words, complete
+    in the order of the device's current stream: for a launch on that stream."""
     # Pinned memory is copied in stream order, so that the host does not wait
     # for the work already on the stream; it goes back to PyTorch's pool, which
     # keeps it until the copy is done.  A stream under capture refuses the copy
@@ -222,9 +223,16 @@ def packed_descs(data: torch.Tensor, out: torch.Tensor, sizes, seeds) -> torch.T
     """Device descriptors for segments of `data` shuffled into the same rows of `out`.
 
     Segment t covers rows offsets[t] .. offsets[t] + sizes[t].  The result can
-    be passed to :func:`bshuffle_batched` repeatedly, e.g. inside a captured
-    CUDA graph.
+    be passed to :func:`bshuffle_batched` repeatedly, on any stream, e.g. inside
+    a captured CUDA graph: the call returns when the descriptors have arrived.
     """
+    descs = _packed_descs(data, out, sizes, seeds)
+    torch.cuda.current_stream(data.device).synchronize()
+    return descs
+
+
+def _packed_descs(data: torch.Tensor, out: torch.Tensor, sizes, seeds) -> torch.Tensor:
+    """packed_descs without the wait: for a launch on the current stream."""
     _require_cuda(data, "data")
     if not data.is_contiguous() or not out.is_contiguous() or out.shape != data.shape:
         raise ValueError("data and out must be contiguous tensors of one shape")
@@ -247,7 +255,7 @@ def batched_packed(data: torch.Tensor, sizes, seeds, rounds: int = DEFAULT_ROUND
     _require_cuda(data, "data")
     data = data.contiguous()
     out = _out_like(data, out)
-    d = packed_descs(data, out, sizes, seeds)
+    d = _packed_descs(data, out, sizes, seeds)
     bshuffle_batched(d.data_ptr(), len(d), row_bytes(data), rounds, _stream_of(data))
     return out
 
