@@ -363,7 +363,8 @@ int bshuffle_release_workspaces(void);
  *       Workspace 2^k * (4 + elem_bytes) bytes plus a little.
  *       bshuffle_inverse of those lengths walks the domain in order instead
  *       (a look-back gives each chunk's first source slot) and buckets by
- *       output window; workspace n * (4 + elem_bytes) bytes plus a little.
+ *       output window; workspace n * (4 + elem_bytes) bytes plus a little,
+ *       and where that cannot be had the single pass runs.
  *   BSHUFFLE_STRATEGY_PIPELINED  the single pass with its look-back taken
  *       off the compute warps, for gathers and scatters of 1, 2, 4, 8 and
  *       16-byte elements and for indices (rows run the plain single pass):

@@ -504,8 +504,9 @@ int bshuffle_inverse(const void *in, void *out, uint64_t n, uint32_t elem_bytes,
         (staged_eligible(n, elem_bytes) || ranked_eligible(n, elem_bytes)) &&
         (strategy == BSHUFFLE_STRATEGY_STAGED || staged_inverse_by_default(geometry_of(n), elem_bytes))) {
         rc = run_staged(in, out, n, elem_bytes, seed, rounds, stream, true);
-        if (rc == BSHUFFLE_OK || strategy == BSHUFFLE_STRATEGY_STAGED) return rc;
-        // auto: the staged buffers could not be had; the single pass needs none
+        if (rc == BSHUFFLE_OK || (strategy == BSHUFFLE_STRATEGY_STAGED && staged_eligible(n, elem_bytes))) return rc;
+        // the staged buffers could not be had; the single pass needs none (and
+        // serves lengths other than 2^k whatever the strategy)
     }
     return run_fused(in, out, n, elem_bytes, seed, rounds, Mode::Scatter, stream);
 }
