@@ -118,8 +118,9 @@ Geometry geometry_of(uint64_t n)
 struct Workspace {
     void *base = nullptr;
     uint64_t status_words = 0;
-    void *aux = nullptr;       // batched plan tables
+    void *aux = nullptr;       // batched look-back ring and plan tables
     size_t aux_bytes = 0;
+    uint32_t batch_tag = 1;    // of the next header: above every tag in the ring
     void *staged = nullptr;    // staged-path buffers
     size_t staged_bytes = 0;
     cudaEvent_t marks[3] = {};  // per-pass timing of the last permute (when enabled)
@@ -177,12 +178,13 @@ int acquire_workspace(cudaStream_t stream, uint64_t words, Workspace **out)
     const uint64_t cap_words = round_up_pow2(words < kMinStatusWords ? kMinStatusWords : words);
     WsHeader keep{};
     keep.tag = 1;
-    keep.batch_tag = 1;
+    keep.batch_tag = ws.batch_tag;
     if (ws.base != nullptr) {
         e = cudaStreamSynchronize(stream);
         if (e != cudaSuccess) return cuda_fail(e);
         e = cudaMemcpy(&keep, ws.base, sizeof(keep), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(e);
+        ws.batch_tag = keep.batch_tag;  // the ring outlives this header, also where the next one cannot be had
         cudaFree(ws.base);
         ws.base = nullptr;
         ws.status_words = 0;
