@@ -9,12 +9,12 @@
 // with earlier steps are the set bits above the element in a shared-memory
 // bitmap of the values seen (a count of the words above it and a population
 // count of its own word), those inside the step come from one ballot per
-// value bit.  About 75 warp instructions per 32 elements, so n^2 / 32 bit
-// operations in all where comparing every pair in shared memory took n^2 / 2
-// comparisons and was bound by the shared-memory loads (96 % busy): 50,000
-// pairs of length 1000 on GB300: 5.53 -> 0.47 ms.
+// value bit.  A step recounts the bitmap, a word a lane: n / 32 steps and about
+// n^2 / 1024 word counts a pair, where comparing every pair in shared memory
+// took n^2 / 2 comparisons and was bound by the shared-memory loads (96 %
+// busy): 50,000 pairs of length 1000 on GB300: 5.53 -> 0.47 ms.
 // Rows that are not permutations of [0, n) have no such sequence: their pairs
-// are marked and counted by the all-pairs kernel, one CTA each.
+// are marked and counted by the all-pairs kernel, a CTA per pair at a time.
 #include <atomic>
 #include <cstdint>
 
@@ -123,19 +123,32 @@ __global__ void __launch_bounds__(kKBlock) kendall_inversions_kernel(const uint3
 }
 
 // Every pair i < j compared, for the pairs of rows marked as no permutations.
+// CTA c owns the pairs c, c + gridDim.x, ..., so that marked pairs which follow
+// one another (all of them, where the rows have ties) run on as many CTAs; one
+// strided load per thread finds the marks of 256 of them at a time.  (With 256
+// consecutive pairs a CTA, 256 marked ones of length 1000 took 6.0 ms.)
 __global__ void __launch_bounds__(kKBlock) kendall_pairs_kernel(const uint32_t *__restrict__ perms, uint32_t n,
                                                                 uint64_t pairs, uint64_t *__restrict__ out)
 {
     __shared__ uint32_t s_a[kMaxN];
     __shared__ uint32_t s_b[kMaxN];
     __shared__ unsigned long long s_sum[kKBlock / 32];
+    __shared__ uint32_t s_marked[kKBlock / 32];  // a bit per pair of the 256
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    for (uint64_t p0 = uint64_t{blockIdx.x} * kKBlock; p0 < pairs; p0 += uint64_t{gridDim.x} * kKBlock) {
-        const bool marked = p0 + tid < pairs && out[p0 + tid] == kNotPermutations;
+    const uint64_t step = gridDim.x;
+    for (uint64_t p0 = blockIdx.x; p0 < pairs; p0 += kKBlock * step) {
+        const uint64_t mine = p0 + tid * step;
+        const bool marked = mine < pairs && out[mine] == kNotPermutations;
+        const uint32_t ball = __ballot_sync(kFull, marked);
+        if (lane == 0) s_marked[warp] = ball;
         if (!__syncthreads_or(marked)) continue;
-        const uint64_t p1 = p0 + kKBlock < pairs ? p0 + kKBlock : pairs;
-        for (uint64_t p = p0; p < p1; ++p) {
-            if (!__syncthreads_or(marked && p == p0 + tid)) continue;
+        // a word of marks and the bit taken from it: the same for the whole CTA
+        uint32_t word = 0, bits = s_marked[0];
+        while (true) {
+            while (bits == 0u && ++word < kKBlock / 32) bits = s_marked[word];
+            if (bits == 0u) break;
+            const uint64_t p = p0 + (word * 32u + static_cast<uint32_t>(__ffs(bits)) - 1u) * step;
+            bits &= bits - 1u;
             const uint32_t *a = perms + 2 * p * n;
             const uint32_t *b = a + n;
             for (uint32_t i = tid; i < n; i += kKBlock) {
@@ -166,6 +179,7 @@ __global__ void __launch_bounds__(kKBlock) kendall_pairs_kernel(const uint32_t *
             }
             __syncthreads();
         }
+        __syncthreads();  // the marks are read before the next ones are written
     }
 }
 
@@ -322,9 +336,8 @@ cudaError_t launch_kendall_pairs(const uint32_t *perms, uint32_t n, uint64_t pai
                                 kKWarps * kendall_warp_bytes(n), stream>>>(perms, n, value_bits, pairs, out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const uint64_t checks = (pairs + kKBlock - 1) / kKBlock;
-    kendall_pairs_kernel<<<static_cast<unsigned>(checks < most ? checks : most), kKBlock, 0, stream>>>(perms, n, pairs,
-                                                                                                      out);
+    kendall_pairs_kernel<<<static_cast<unsigned>(pairs < most ? pairs : most), kKBlock, 0, stream>>>(perms, n, pairs,
+                                                                                                    out);
     return cudaGetLastError();
 }
 
