@@ -19,7 +19,9 @@ default strategy runs that kernel, and the fastest is selected:
 Every configuration computes the same output; only speed differs.  Results
 are cached as JSON keyed by device name, compute capability and SM count,
 then kernel and element width; `apply_cached()` re-selects the cached
-choices in a new process.
+choices in a new process.  A choice is cached with its shape, and passed over
+where the library's configuration of that number has another one (or the file
+names none): it was timed on a kernel that is no longer there.
 """
 from __future__ import annotations
 
@@ -80,16 +82,21 @@ def _time_ms(fn, reps: int, warmup: int, calls: int = 1) -> float:
     return statistics.median(times)
 
 
+def _shape(described: dict) -> dict:
+    return {k: v for k, v in described.items() if k != "config"}
+
+
 def _sweep(kernel: int, width: int, fn, rounds: int, reps: int, warmup: int, calls: int = 1) -> dict:
-    timings = {}
+    timings, shapes = {}, {}
     for c in _lib.bshuffle_kernel_configs(kernel):
         if c["rounds_unrolled"] not in (0, rounds) and kernel == _lib.BSHUFFLE_KERNEL_SINGLE_PASS:
             continue  # a fixed round count that this call does not use
         _lib.bshuffle_kernel_select(kernel, width, c["config"])
         timings[c["config"]] = _time_ms(fn, reps, warmup, calls)
+        shapes[c["config"]] = _shape(c)
     best = min(timings, key=timings.get)
     _lib.bshuffle_kernel_select(kernel, width, best)
-    return {"config": best, "ms": {str(k): v for k, v in timings.items()}}
+    return {"config": best, "shape": shapes[best], "ms": {str(k): v for k, v in timings.items()}}
 
 
 def tune(widths=WIDTHS, kernels=tuple(KERNELS), rounds: int = 24, reps: int = 5, warmup: int = 2,
@@ -147,7 +154,8 @@ def tune(widths=WIDTHS, kernels=tuple(KERNELS), rounds: int = 24, reps: int = 5,
 
 
 def apply_cached(cache: str = CACHE) -> bool:
-    """Select the cached configurations for the current device; False if none."""
+    """Select the cached configurations for the current device; False if there
+    are none that the library still has."""
     if not os.path.exists(cache):
         return False
     with open(cache) as fh:
@@ -155,12 +163,16 @@ def apply_cached(cache: str = CACHE) -> bool:
     entry = data.get(device_key())
     if not entry:
         return False
+    applied = False
     for kernel, per_width in entry.items():
         if kernel not in KERNELS:
             continue
+        shapes = {c["config"]: _shape(c) for c in _lib.bshuffle_kernel_configs(KERNELS[kernel])}
         for w, rec in per_width.items():
-            _lib.bshuffle_kernel_select(KERNELS[kernel], int(w), int(rec["config"]))
-    return True
+            if "shape" in rec and rec["shape"] == shapes.get(int(rec["config"])):
+                _lib.bshuffle_kernel_select(KERNELS[kernel], int(w), int(rec["config"]))
+                applied = True
+    return applied
 
 
 def reset() -> None:
