@@ -7,10 +7,10 @@ is timed with CUDA events on the current stream, at the size class where the
 default strategy runs that kernel, and the fastest is selected:
 
 * the plain single-pass kernel (BSHUFFLE_KERNEL_SINGLE_PASS) on a domain of
-  2^17 (n = 2^16 + 1): below 2^18 domain indices the default runs it, and a
+  2^17 (n = 2^16 + 1): below 2^20 domain indices the default runs it, and a
   call is all latency, so a timing is a run of back-to-back calls;
 * the pipelined single pass (BSHUFFLE_KERNEL_PIPELINED) at n = 2^24 + 1
-  (domain 2^25): from 2^18 domain indices up to the staged path's size, and
+  (domain 2^25): from 2^20 domain indices up to the staged path's size, and
   for 16-byte elements of any larger length;
 * the persistent batched kernel (BSHUFFLE_KERNEL_BATCHED) on an uneven batch
   of independent shuffles with log-uniform sizes in [100, 2,000,000] (4,096

@@ -62,15 +62,18 @@ bool staged_inverse_by_default(const Geometry &g, uint32_t elem_bytes)
     if (elem_bytes == 16) return mostly_kept && bytes >= 224 * kMiB;
     return bytes >= kStagedMinBytes || (mostly_kept && bytes >= 126 * kMiB);
 }
-// Auto strategy: the pipelined single pass from these domain exponents on.
-// On smaller domains a launch is all latency, and the plain kernel, without
-// the hand-offs between compute warps and look-back warp, finishes first:
-// back-to-back calls at n = 2^m + 1 (4, 8 and 16-byte elements, GB300) took
-// ~8.2 us plain against ~10.2 us pipelined up to m = 14, and the pipelined
-// kernel first won at a 2^18 domain for gathers and indices and at 2^19 for
-// the scatter of bshuffle_inverse.
-constexpr uint32_t kPipeMinKGather = 18;
-constexpr uint32_t kPipeMinKScatter = 19;
+// Auto strategy: the pipelined single pass from this domain exponent on.  On
+// smaller domains a launch is all latency, and the plain kernel, without the
+// hand-offs between compute warps and look-back warp, finishes first.  Calls
+// replayed from a graph on GB300, plain / pipelined, us: 2-byte gathers at 2^17
+// + 1 8.0 / 9.7, 2^19 + 1 12.3 / 13.9, 2^20 - 1 12.4 / 15.7, 1,200,007 25.8 /
+// 26.9, 2^21 + 1 38.1 / 31.9; 4-byte at 2^17 + 1 8.4 / 8.9, 2^18 + 1 10.5 /
+// 12.0, 2^19 + 1 12.4 / 12.5, 2^20 - 1 13.5 / 12.8; 64-bit indices at 2^19 + 1
+// 12.1 / 13.3, 2^20 - 1 12.6 / 13.8, 2^20 + 1 25.1 / 21.6; 8-byte scatters at
+// 2^18 + 1 11.8 / 13.4, 2^19 + 1 13.8 / 15.4, 2^20 - 1 16.4 / 17.5, 1-byte at
+// 2^19 + 1 15.5 / 16.0, 2^20 + 1 31.1 / 27.7.  With 10 rounds the plain kernel
+// gains a little more at 2^17 + 1 (4-byte gathers 7.8 / 8.7).
+uint32_t pipe_min_k(Mode mode, uint32_t elem_bytes) { return mode == Mode::Gather && elem_bytes >= 4 ? 20 : 21; }
 
 // ------------------------------------------------------------------ host math
 
@@ -295,8 +298,8 @@ int run_fused(const void *in, void *out, uint64_t n, uint32_t elem_bytes, uint64
         return BSHUFFLE_OK;
     }
     // the pipelined kernel: on request for every call it serves, and by
-    // default for those over domains of at least 2^18 (2^19 for the scatter)
-    const bool pipe_by_default = a.g.k >= (mode == Mode::Scatter ? kPipeMinKScatter : kPipeMinKGather);
+    // default for those over large enough domains
+    const bool pipe_by_default = a.g.k >= pipe_min_k(mode, elem_bytes);
     const bool pipe = !rows && bsh::pipe_supports(mode, elem_bytes) &&
                       (which == FusedKernel::Pipelined ||
                        (which == FusedKernel::ByStrategy &&
