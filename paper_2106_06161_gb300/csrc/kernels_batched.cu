@@ -271,7 +271,7 @@ __device__ __forceinline__ void resolve_job(const BatchArgs &a, uint32_t ticket,
 // only after the look-back: a CTA that held a ticket while its current tile
 // still waited on other tiles would make every later tile wait for it.  Warp
 // 1 takes it and resolves it into buffer b ^ 1 while the other warps store.
-template <class T, bool ODD, int ITEMS, int ENTRIES>
+template <class T, bool ODD, int ITEMS, int ENTRIES, bool UNROLL>
 __device__ __forceinline__ void batch_tile(const BatchArgs &a, const BatchJob &job, BatchShared<ENTRIES> &sh, int b,
                                            const dev::StatusRing &ring, uint64_t total)
 {
@@ -290,7 +290,10 @@ __device__ __forceinline__ void batch_tile(const BatchArgs &a, const BatchJob &j
         left[j] = i >> g.R;
         right[j] = i & g.rmask;
     }
-    dev::cipher_items<ODD, ITEMS>(left, right, sh.keys[b], a.rounds, g);
+    if constexpr (UNROLL)
+        dev::cipher_items<ODD, ITEMS>(left, right, sh.keys[b], a.rounds, g);
+    else
+        dev::cipher_items_loop<ODD, ITEMS>(left, right, sh.keys[b], a.rounds, g);
     uint32_t src[ITEMS];
     bool keep[ITEMS];
     T val[ITEMS];
@@ -336,7 +339,10 @@ __device__ __forceinline__ void batch_tile(const BatchArgs &a, const BatchJob &j
 // are ready to start the tile, so the smallest unfinished ticket always
 // belongs to a running CTA whose look-back depends only on smaller tickets:
 // every wait ends.
-template <class T>
+// UNROLL: for the default 24 rounds; other counts have an instance of their
+// own, without the 24-round forms, whose registers made it spill (512 uneven
+// instances of 1-byte elements with 10 rounds 540 -> 485 us).
+template <class T, bool UNROLL>
 __global__ void __launch_bounds__(kBBlock, min_ctas_for(sizeof(T))) batch_tile_kernel(const __grid_constant__ BatchArgs a)
 {
     constexpr int ENTRIES = kBItems * (kBBlock / 32);
@@ -355,9 +361,9 @@ __global__ void __launch_bounds__(kBBlock, min_ctas_for(sizeof(T))) batch_tile_k
         const BatchJob job = sh.job[b];
         if (job.ticket >= total) break;
         if (job.g.k & 1u)
-            batch_tile<T, true, kBItems, ENTRIES>(a, job, sh, b, ring, total);
+            batch_tile<T, true, kBItems, ENTRIES, UNROLL>(a, job, sh, b, ring, total);
         else
-            batch_tile<T, false, kBItems, ENTRIES>(a, job, sh, b, ring, total);
+            batch_tile<T, false, kBItems, ENTRIES, UNROLL>(a, job, sh, b, ring, total);
     }
     if (threadIdx.x == 0) finish_batch(a, ring, total);
 }
@@ -660,8 +666,8 @@ cudaError_t launch_pipe_typed(const BatchArgs &a, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t launch_typed(const BatchArgs &a, cudaStream_t stream)
+template <class T, bool UNROLL>
+cudaError_t launch_rounds(const BatchArgs &a, cudaStream_t stream)
 {
     static std::atomic<int> per_sm[64];  // CTAs to launch per device, 0 until first use
     int device = 0;
@@ -671,7 +677,7 @@ cudaError_t launch_typed(const BatchArgs &a, cudaStream_t stream)
     int ctas_cached = per_sm[device].load(std::memory_order_acquire);
     if (ctas_cached == 0) {
         int blocks = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, batch_tile_kernel<T>, kBBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, batch_tile_kernel<T, UNROLL>, kBBlock, 0);
         if (e != cudaSuccess) return e;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
@@ -684,8 +690,14 @@ cudaError_t launch_typed(const BatchArgs &a, cudaStream_t stream)
     batch_plan_kernel<<<1, kPlanThreads, 0, stream>>>(b);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    batch_tile_kernel<T><<<b.grid, kBBlock, 0, stream>>>(b);
+    batch_tile_kernel<T, UNROLL><<<b.grid, kBBlock, 0, stream>>>(b);
     return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_typed(const BatchArgs &a, cudaStream_t stream)
+{
+    return a.rounds == dev::kUnrolledRounds ? launch_rounds<T, true>(a, stream) : launch_rounds<T, false>(a, stream);
 }
 
 template <class T>
