@@ -367,23 +367,10 @@ __device__ __forceinline__ void cipher_inverse_items_loop(uint32_t (&left)[ITEMS
     for (int j = 0; j < ITEMS; ++j) right[j] &= g.rmask;
 }
 
-template <bool ODD, int ITEMS, int ROUNDS>
-__device__ __forceinline__ void cipher_inverse_items_fixed(uint32_t (&left)[ITEMS], uint32_t (&right)[ITEMS],
-                                                           const uint32_t *keys, const Geometry &g)
-{
-#pragma unroll
-    for (int r = ROUNDS - 1; r >= 0; --r) {
-#pragma unroll
-        for (int j = 0; j < ITEMS; ++j) cipher_inverse_round<ODD>(left[j], right[j], keys[r], g.lift_mul, g.lmask);
-    }
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) right[j] &= g.rmask;
-}
-
 // Default rounds: the high product word without its 32 x 32 -> 64-bit
 // product (four of the even round's eight issue cycles on the FMA-heavy pipe,
-// of the odd one's ten).  As
-// in cipher_items_float the left half is kept as X = 2^23 + left, and the high
+// of the odd one's ten).  As in cipher_items_float the left half is kept as
+// X = 2^23 + left, and the high
 // word's low L bits are left * (M0hi - 1) + floor(left * 1.694...), now for
 // every L up to 16: the multiplier (2^32 + M0lo) / 2^32 is split into 217 / 128
 // (2^23 of it is a multiple of 2^16, so that the pattern adds nothing below bit
@@ -391,8 +378,9 @@ __device__ __forceinline__ void cipher_inverse_items_fixed(uint32_t (&left)[ITEM
 // floor (the first one's value is rounded to a grid that holds the multiples of
 // 2^-7 at which the second one's floor steps).  The forward round gains nothing
 // from this (its product gives the low word too).  MIXED: at most 12 bits, one
-// FMA.  Measured on GB300, 2^28 evaluations at k = 28: 1.35 -> 1.15 ms; the shuffle of 2^27 4-byte elements
-// (odd k) 1.80 -> 1.71 ms, of 2^27 - 5 8-byte ones 2.38 -> 2.32.
+// FMA.  Measured on GB300, 2^28 evaluations at k = 28: 1.35 -> 1.15 ms; the
+// shuffle of 2^27 4-byte elements (odd k) 1.80 -> 1.71 ms, of 2^27 - 5 8-byte
+// ones 2.38 -> 2.32.
 constexpr float kFracTop = 217.0f / 128.0f;
 constexpr float kFracRest = -(static_cast<float>(0xB2000000u - kM0Lo) / 4294967296.0f);
 static_assert(0xB2000000u - kM0Lo < (1u << 22), "the rest of the multiplier is exact in a float");
@@ -572,10 +560,10 @@ __device__ __forceinline__ uint32_t warp_inclusive_scan(uint32_t v)
 // Where the tile-status words of a launch live and how they are tagged.
 // Tile q's word is words[q & mask] and carries tag base_tag + (q >> shift).
 // A plain launch uses one word per tile (mask = all ones, shift = 63) and the
-// launch tag; the persistent batched launch reuses a ring of 2^shift words,
-// cleared at the start of the launch, and tags each pass over the ring with
-// its generation so that a word left by tile q - 2^shift never reads as
-// tile q's.
+// launch tag; the persistent batched launch reuses a ring of 2^shift words and
+// tags each pass over the ring with its generation, counted on from the
+// launches before it on the stream, so that neither a word left by tile
+// q - 2^shift nor one of an earlier launch ever reads as tile q's.
 struct StatusRing {
     uint64_t *words;
     uint64_t mask;

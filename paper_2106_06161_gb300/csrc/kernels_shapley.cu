@@ -32,7 +32,7 @@ using dev::kFull;
 constexpr int kSvBlock = 256;
 constexpr int kSvWarps = kSvBlock / 32;
 constexpr int kSvItems = 8;
-constexpr int kSvGroup = 4;  // indices that share the cipher's first round (from 2^14 players on)
+constexpr int kSvGroup = 4;  // indices that share the cipher's first round (from 8,193 players on)
 constexpr uint32_t kSvChunk = 32 * kSvItems;
 
 template <bool ODD, CipherForm FORM>

@@ -18,15 +18,20 @@
 //     slots (scatter: read those slots and write them to the images).
 //   look-back warp, tile i: wait for the counts, form the parts' offsets,
 //     look back, publish the inclusive prefix and hand the prefix to the
-//     compute warps; then take the ticket of tile i + 2.
+//     compute warps; then take the ticket of tile i + 2 (the second ticket,
+//     once the first tile is published).  Launches over kTicketsAheadBytes: the
+//     last compute warp takes the ticket of tile i + 1 instead, when the stores
+//     of tile i - 1 are done; the look-back of tile i may still be running.
 //
 // The compute warps share no barrier and pass on as soon as the ticket and
-// the rank that they need are there.  Tickets stay in order of readiness: a
-// ticket is taken only when the CTA's latest look-back is over (the second
-// one, once its first tile is published), and a tile's aggregate is published
-// by the compute warps right after its counts, never after a later look-back.
-// The smallest unfinished ticket therefore always makes progress.  Every wait
-// is bounded.
+// the rank that they need are there.  When a ticket is taken, nothing is left
+// that its tile's aggregate would have to wait for: ahead, the compute warps
+// are at most in tile i + 1, whose stores of tile i need the look-back that is
+// over; else they are at the end of tile i.  They publish the aggregate right
+// after the tile's counts, so every ticket's aggregate comes without waiting
+// for a look-back of any CTA, a look-back waits for aggregates of smaller
+// tickets only, and the smallest unfinished ticket always makes progress.
+// Every wait is bounded.
 //
 // What bounds it: up to the L2's size the ALU pipe (cipher) and, below some
 // 2^20 indices, the latency of one tile's steps; beyond, the random-access
