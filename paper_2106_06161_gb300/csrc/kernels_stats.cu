@@ -14,7 +14,8 @@
 // took n^2 / 2 comparisons and was bound by the shared-memory loads (96 %
 // busy): 50,000 pairs of length 1000 on GB300: 5.53 -> 0.47 ms.
 // Rows that are not permutations of [0, n) have no such sequence: their pairs
-// are marked and counted by the all-pairs kernel, a CTA per pair at a time.
+// are marked and counted by the all-pairs kernel, a CTA per pair at a time,
+// which also serves few short rows (all_pairs_by_default).
 #include <atomic>
 #include <cstdint>
 
@@ -122,65 +123,94 @@ __global__ void __launch_bounds__(kKBlock) kendall_inversions_kernel(const uint3
     }
 }
 
-// Every pair i < j compared, for the pairs of rows marked as no permutations.
+// Every pair i < j compared: all pairs of rows (ALL), or those marked as no
+// permutations.
 // CTA c owns the pairs c, c + gridDim.x, ..., so that marked pairs which follow
 // one another (all of them, where the rows have ties) run on as many CTAs; one
 // strided load per thread finds the marks of 256 of them at a time.  (With 256
 // consecutive pairs a CTA, 256 marked ones of length 1000 took 6.0 ms.)
+struct KendallShared {
+    uint32_t a[kMaxN];
+    uint32_t b[kMaxN];
+    unsigned long long sum[kKWarps];
+    uint32_t marked[kKWarps];  // a bit per pair of 256
+};
+
+// Pair p by the whole CTA.
+__device__ __forceinline__ void count_all_pairs(const uint32_t *__restrict__ perms, uint32_t n, uint64_t p,
+                                                uint64_t *__restrict__ out, KendallShared &sh)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t *a = perms + 2 * p * n;
+    const uint32_t *b = a + n;
+    for (uint32_t i = tid; i < n; i += kKBlock) {
+        sh.a[i] = a[i];
+        sh.b[i] = b[i];
+    }
+    __syncthreads();
+    unsigned long long count = 0;
+    // rows i and n-1-i together keep the work per thread balanced
+    for (uint32_t i = tid; i < (n + 1) / 2; i += kKBlock) {
+        for (uint32_t r = 0; r < 2; ++r) {
+            const uint32_t row = r == 0 ? i : n - 1 - i;
+            if (r == 1 && row == i) break;
+            const uint32_t ai = sh.a[row], bi = sh.b[row];
+            uint32_t c = 0;
+            for (uint32_t j = row + 1; j < n; ++j) c += ((ai < sh.a[j]) != (bi < sh.b[j])) ? 1u : 0u;
+            count += c;
+        }
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) count += __shfl_down_sync(kFull, count, d);
+    if (lane == 0) sh.sum[warp] = count;
+    __syncthreads();
+    if (tid == 0) {
+        unsigned long long total = 0;
+        for (int w = 0; w < kKWarps; ++w) total += sh.sum[w];
+        out[p] = total;
+    }
+    __syncthreads();
+}
+
+template <bool ALL>
 __global__ void __launch_bounds__(kKBlock) kendall_pairs_kernel(const uint32_t *__restrict__ perms, uint32_t n,
                                                                 uint64_t pairs, uint64_t *__restrict__ out)
 {
-    __shared__ uint32_t s_a[kMaxN];
-    __shared__ uint32_t s_b[kMaxN];
-    __shared__ unsigned long long s_sum[kKBlock / 32];
-    __shared__ uint32_t s_marked[kKBlock / 32];  // a bit per pair of the 256
+    __shared__ KendallShared sh;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint64_t step = gridDim.x;
+    if constexpr (ALL) {
+        for (uint64_t p = blockIdx.x; p < pairs; p += step) count_all_pairs(perms, n, p, out, sh);
+        return;
+    }
     for (uint64_t p0 = blockIdx.x; p0 < pairs; p0 += kKBlock * step) {
         const uint64_t mine = p0 + tid * step;
         const bool marked = mine < pairs && out[mine] == kNotPermutations;
         const uint32_t ball = __ballot_sync(kFull, marked);
-        if (lane == 0) s_marked[warp] = ball;
+        if (lane == 0) sh.marked[warp] = ball;
         if (!__syncthreads_or(marked)) continue;
         // a word of marks and the bit taken from it: the same for the whole CTA
-        uint32_t word = 0, bits = s_marked[0];
+        uint32_t word = 0, bits = sh.marked[0];
         while (true) {
-            while (bits == 0u && ++word < kKBlock / 32) bits = s_marked[word];
+            while (bits == 0u && ++word < kKWarps) bits = sh.marked[word];
             if (bits == 0u) break;
-            const uint64_t p = p0 + (word * 32u + static_cast<uint32_t>(__ffs(bits)) - 1u) * step;
+            count_all_pairs(perms, n, p0 + (word * 32u + static_cast<uint32_t>(__ffs(bits)) - 1u) * step, out, sh);
             bits &= bits - 1u;
-            const uint32_t *a = perms + 2 * p * n;
-            const uint32_t *b = a + n;
-            for (uint32_t i = tid; i < n; i += kKBlock) {
-                s_a[i] = a[i];
-                s_b[i] = b[i];
-            }
-            __syncthreads();
-            unsigned long long count = 0;
-            // rows i and n-1-i together keep the work per thread balanced
-            for (uint32_t i = tid; i < (n + 1) / 2; i += kKBlock) {
-                for (uint32_t r = 0; r < 2; ++r) {
-                    const uint32_t row = r == 0 ? i : n - 1 - i;
-                    if (r == 1 && row == i) break;
-                    const uint32_t ai = s_a[row], bi = s_b[row];
-                    uint32_t c = 0;
-                    for (uint32_t j = row + 1; j < n; ++j) c += ((ai < s_a[j]) != (bi < s_b[j])) ? 1u : 0u;
-                    count += c;
-                }
-            }
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) count += __shfl_down_sync(kFull, count, d);
-            if (lane == 0) s_sum[warp] = count;
-            __syncthreads();
-            if (tid == 0) {
-                unsigned long long total = 0;
-                for (int w = 0; w < kKBlock / 32; ++w) total += s_sum[w];
-                out[p] = total;
-            }
-            __syncthreads();
         }
         __syncthreads();  // the marks are read before the next ones are written
     }
+}
+
+// Comparing every pair takes one launch and no bitmap: faster for few short
+// rows.  Calls replayed from a graph on GB300, all pairs / inversions, us: n =
+// 32, 600 pairs 2.6 / 3.9, 1,200 4.3 / 4.5, 2,500 7.1 / 5.2; n = 100, 600 3.7 /
+// 6.4, 1,200 6.4 / 7.0; n = 200, 600 6.2 / 7.9, 1,200 10.4 / 8.6; n = 300, 300
+// 6.6 / 10.0, 600 9.8 / 10.1, 1,200 16.7 / 10.7; n = 400, 100
+// 6.9 / 11.8, 300 9.2 / 11.9, 600 15.1 / 12.0; n = 600 (a thread then has
+// several rows), 16 15.5 / 16.3, 300 19.2 / 16.5.
+bool all_pairs_by_default(uint32_t n, uint64_t pairs, uint64_t resident)
+{
+    return n <= 2 * kKBlock && pairs <= resident && pairs * n <= 180'000u;
 }
 
 // Row r of `sigma` = the ranks of the shuffle with seed seed0 + r:
@@ -321,6 +351,12 @@ cudaError_t launch_kendall_pairs(const uint32_t *perms, uint32_t n, uint64_t pai
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
     if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
+    const uint64_t most = static_cast<uint64_t>(sms) * 8;
+    const unsigned grid = static_cast<unsigned>(pairs < most ? pairs : most);
+    if (all_pairs_by_default(n, pairs, most)) {
+        kendall_pairs_kernel<true><<<grid, kKBlock, 0, stream>>>(perms, n, pairs, out);
+        return cudaGetLastError();
+    }
     static std::atomic<bool> configured[64];  // attribute set on this device
     if (!configured[device].load(std::memory_order_acquire)) {
         e = cudaFuncSetAttribute(kendall_inversions_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -330,14 +366,12 @@ cudaError_t launch_kendall_pairs(const uint32_t *perms, uint32_t n, uint64_t pai
     }
     uint32_t value_bits = 0;
     while ((1u << value_bits) < n) ++value_bits;
-    const uint64_t most = static_cast<uint64_t>(sms) * 8;
     const uint64_t blocks = (pairs + kKWarps - 1) / kKWarps;
     kendall_inversions_kernel<<<static_cast<unsigned>(blocks < most ? blocks : most), kKBlock,
                                 kKWarps * kendall_warp_bytes(n), stream>>>(perms, n, value_bits, pairs, out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    kendall_pairs_kernel<<<static_cast<unsigned>(pairs < most ? pairs : most), kKBlock, 0, stream>>>(perms, n, pairs,
-                                                                                                    out);
+    kendall_pairs_kernel<false><<<grid, kKBlock, 0, stream>>>(perms, n, pairs, out);
     return cudaGetLastError();
 }
 
