@@ -45,7 +45,8 @@ template <class T, Mode MODE, int BLOCK>
 constexpr int kElemMinCtas = MODE == Mode::Gather && sizeof(T) <= 2 && BLOCK == 256 ? 6 : 0;
 
 template <class T, Mode MODE, bool ODD, int BLOCK, int ITEMS, int ROUNDS, int BIJ = kVarPhilox, bool RANGE = false>
-__global__ void __launch_bounds__(BLOCK, kElemMinCtas<T, MODE, BLOCK>) elem_tile_kernel(const __grid_constant__ TileArgs a)
+__global__ void __launch_bounds__(BLOCK, kElemMinCtas<T, MODE, BLOCK>)
+elem_tile_kernel(const __grid_constant__ TileArgs a)
 {
     constexpr int WARPS = BLOCK / 32;
     constexpr int ENTRIES = ITEMS * WARPS;
