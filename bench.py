@@ -293,17 +293,22 @@ def traffic_for(kernel: str, fingerprint: str):
     return rec.get("dram_bytes_per_launch")
 
 
-# Pass 1 of the staged path is bound by integer issue: 2^28 inverse cipher
+# Pass 1 of the staged path is bound by instruction issue: 2^28 inverse cipher
 # evaluations per launch.  ncu on that kernel (n = 2^26 uint64, even k) puts
-# the FMA-heavy pipe, which issues the integer multiplies, at the top of the
-# pipes (sm__pipe_fmaheavy_cycles_active); its peak rate is one warp
-# instruction every two cycles per SM sub-partition (16 lanes).  The derived
-# peak is the evaluation rate at which that pipe is busy every cycle:
+# the FMA-heavy pipe, which issues the integer multiply-adds and the paired
+# single-precision FMAs, at the top of the pipes (70 % busy, the ALU pipe 69 %);
+# its peak rate is one warp instruction every two cycles per SM sub-partition
+# (16 lanes).  The derived peak is the evaluation rate at which that pipe is
+# busy every cycle:
 #   152 SMs x 4 sub-partitions x 16 lanes x 2.07 GHz
 #   / (FMA-heavy thread instructions per evaluation, counted by ncu as
 #      smsp__inst_executed_pipe_fmaheavy.sum x 32 / evaluations).
 SMS, SMSP_PER_SM, FMAHEAVY_LANES, SM_HZ = 152, 4, 16, 2.07e9
-FMAHEAVY_INST_PER_INVERSE_EVAL = 80.1  # ncu, n = 2^26 uint64: 72 multiplies + 8 of addressing
+# ncu, n = 2^26 uint64: per round two integer multiply-adds and two FMAs that two
+# evaluations share, so 72, + 8 of addressing
+FMAHEAVY_INST_PER_INVERSE_EVAL = 80.5
+# The output window of pass 2 at the main workload: 4 MiB, 2^19 uint64.
+MAIN_WINDOW_LOG2 = 19
 
 
 def alu_peak_evals_per_s() -> float:
@@ -319,8 +324,8 @@ def roofline_for(passes, bsbuild, strategy, window_scatter_ms=None, step_ms=None
     read by pass 2: 20 B per uint64 element and pass) is reported beside it,
     not as algorithmic.  The staged scatter pass also gets its fraction of
     the window-scatter kernel (the same sequential reads and random writes
-    into 8 MiB windows with nothing else), the L2 random-write ceiling it
-    runs into."""
+    into windows of the same size, with nothing else), the L2 random-write
+    ceiling it runs into."""
     peak, peak_kind = measured_peaks()
     n = N_MAIN
     algo = 2 * n * ELEM
@@ -432,8 +437,8 @@ def run_ours(args):
         src = bs.indices(N_MAIN, seed)[idx]
         assert torch.equal(y[idx], x[src]), "shuffle output does not match its index sequence"
     # the ceiling of the staged scatter pass, live: sequential reads and
-    # random writes inside 8 MiB windows (2^20 uint64), nothing else
-    ws = lambda: bs.bshuffle_window_scatter(xp, yp, N_MAIN, ELEM, 20, sptr)  # noqa: E731
+    # random writes inside windows of the pass's size, nothing else
+    ws = lambda: bs.bshuffle_window_scatter(xp, yp, N_MAIN, ELEM, MAIN_WINDOW_LOG2, sptr)  # noqa: E731
     for _ in range(3):
         ws()
     _, ws_region = timed_launches(ws, 10, stream, torch)
