@@ -371,7 +371,11 @@ cudaError_t launch_kendall_pairs(const uint32_t *perms, uint32_t n, uint64_t pai
                                 kKWarps * kendall_warp_bytes(n), stream>>>(perms, n, value_bits, pairs, out);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    kendall_pairs_kernel<false><<<grid, kKBlock, 0, stream>>>(perms, n, pairs, out);
+    // half of the CTAs that fit: 0.2 us a call that has nothing marked (0.7 with
+    // all of them, 2,000 pairs of length 1000 31.7 and 32.3 us), and 2,000 pairs
+    // with ties of length 1000 247 us (240)
+    const unsigned check = static_cast<unsigned>(pairs < most / 2 ? pairs : most / 2);
+    kendall_pairs_kernel<false><<<check, kKBlock, 0, stream>>>(perms, n, pairs, out);
     return cudaGetLastError();
 }
 
